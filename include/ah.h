@@ -150,6 +150,15 @@ ah_status ah_ctx_set_timing(ah_ctx* ctx, int enable);
  * context stays usable. */
 ah_status ah_ctx_inject_alloc_failures(ah_ctx* ctx, int n);
 
+/* Generated scan kernels come in two forms that find the same sites.  The shifted form reads each
+ * pattern position from shifted words of the code planes.  The interleaved form transposes tiles of
+ * 32,768 bases so that no word is shifted: it scans 1.6 to 2.2 times as fast, takes two to three times
+ * as long to compile, and needs at least about 512 tiles to fill the GPU.  Plans take the interleaved
+ * form for batches of at least 16.8 Mbp where the primers suit it (at most 32 pairs, and not so many
+ * expected sites that checking them dominates), and otherwise the shifted form, which regular scans
+ * always use.  Setting a shape or a circuit with the two calls below keeps the context's later plans on
+ * the shifted form they describe. */
+
 /* Shape of the scan kernel used by ah_scan_primers on this context (a tuning knob; results do not
  * depend on it): threads per CTA (32..1024, a multiple of 32), groups of 32 positions per thread
  * (1..16), initial site slots per tile (16..4096, a power of two), and how pattern positions are
@@ -527,7 +536,7 @@ typedef struct {
   uint64_t hit_capacity, amp_capacity, arena_capacity; /* 0: sized from an exact run */
 } ah_plan_params;
 typedef struct {
-  int32_t threads, groups_per_thread, shift_mode, persistent, grid;
+  int32_t threads, groups_per_thread, shift_mode, persistent, grid; /* 64 x 32: the interleaved form */
   uint32_t slot_cap, max_tile_sites;
   uint64_t hit_capacity, amp_capacity, arena_capacity;
   uint64_t n_hits, n_amps, n_kept, arena_bytes; /* of the last checked run */

@@ -523,6 +523,7 @@ ah_status ah_ctx_set_scan_config(ah_ctx* ctx, int threads, int groups_per_thread
   if (threads < 32 || threads > 1024 || threads % 32 || groups_per_thread < 1 || groups_per_thread > 16 ||
       slot_cap < 16 || slot_cap > 4096 || (slot_cap & (slot_cap - 1)) || shift_mode < 0 || shift_mode > 2)
     return fail(ctx, AH_EINVAL, "ah_ctx_set_scan_config: values out of range");
+  ctx->scan_cfg_given = true;
   ctx->scan_cfg.threads = threads;
   ctx->scan_cfg.groups_per_thread = groups_per_thread;
   ctx->scan_cfg.slot_cap = slot_cap;
@@ -535,6 +536,7 @@ ah_status ah_ctx_set_scan_circuit(ah_ctx* ctx, int min_blocks, int vote_windows,
   if (min_blocks < 0 || min_blocks > 32 || vote_windows < 1 || vote_windows > (1 << 20) || emit_queue < 0 ||
       emit_queue > 1)
     return fail(ctx, AH_EINVAL, "ah_ctx_set_scan_circuit: values out of range");
+  ctx->scan_cfg_given = true;
   ctx->scan_cfg.min_blocks = min_blocks;
   ctx->scan_cfg.vote_windows = vote_windows;
   ctx->scan_cfg.emit_queue = emit_queue;

@@ -87,7 +87,20 @@ struct ScanConfig {
   int vote_windows = 1024;  // generated kernels: windows the phase-split cost model takes one warp vote
                             // to cover (1024 = 32 lanes x 32 positions on uniform random bases; larger
                             // values weigh phase two as if windows survived phase one more often)
+  int interleaved = 0;      // generated kernels: 1 the interleaved form (see ah_jit.cpp), whose tiles are
+                            // kIlTileGroups groups whatever threads and groups_per_thread say
+  int il_rows = 0;          // interleaved form: positions per loop iteration (0: by the pattern count)
 };
+
+// The interleaved form: a warp takes kIlTileGroups consecutive groups, a block kIlWarps of them.
+constexpr int kIlTileGroups = 1024, kIlWarps = 2;
+// groups per slot-list tile, and groups per block of the generated kernel
+inline uint64_t scan_tile_groups(const ScanConfig& c) {
+  return c.interleaved ? (uint64_t)kIlTileGroups : (uint64_t)c.threads * c.groups_per_thread;
+}
+inline uint64_t scan_block_groups(const ScanConfig& c) {
+  return c.interleaved ? (uint64_t)kIlTileGroups * kIlWarps : (uint64_t)c.threads * c.groups_per_thread;
+}
 
 // default of ah_ctx::tm_split_sites: each launch re-reads the window's site marks, which pays once
 // the chains of fewer primers per launch keep the instruction cache warm
@@ -110,6 +123,7 @@ struct ah_ctx {
   ah::JitCache* jit = nullptr;       // the process-wide kernel cache
   std::mutex stats_mu;               // compile counters are updated from compile threads
   ah::ScanConfig scan_cfg;
+  bool scan_cfg_given = false;       // set by the caller: plans then keep the shifted form it describes
   int sm_count = 0;
   // diagnostics
   uint64_t n_launches = 0;
@@ -369,9 +383,16 @@ void launch_extract(cudaStream_t s, bool write, const ah_amplicon* amps, uint64_
 // ---- run-time specialised scan kernels (ah_jit.cpp) ------------------------------------------
 struct ScanKernel {
   cudaKernel_t fn = nullptr;
-  int threads = 0, groups_per_thread = 0;
+  int threads = 0;
+  uint64_t tile_groups = 0;   // groups per slot-list tile
+  uint64_t block_groups = 0;  // groups per block (one-CTA-per-block forms)
   int alu_ops_per_group = 0;  // LOP3 + funnel-shift instructions of the generated circuit per 32 positions
 };
+// Whether the interleaved form is the faster one for these patterns: at most kIlMaxPatterns of them,
+// and few enough windows pass their filters.  On random bases a set with 36 sites per iteration of the
+// loop (8,192 windows) ran as fast in both forms, one with 95 1.8x slower in the interleaved form; the
+// line is at half the queue, 48.
+bool interleaved_suits(const std::vector<Pattern>& pats);
 std::string scan_source(const std::vector<Pattern>& pats, const ScanConfig& cfg, int* alu_ops_per_group = nullptr);
 // NVRTC for this device's architecture (host work only); fills cubin or returns a message
 ah_status nvrtc_compile(int device, const std::string& src, const char* name, std::vector<char>* cubin,

@@ -363,7 +363,7 @@ PatternCode gen_pattern(Emitter& EA, int* tmp, const Pattern& P, std::map<std::p
   return emit_pattern(EA, tmp, S, choose_split(S, used_a, windows), used_a);
 }
 
-const char* kPrelude = R"(
+const char* kParams = R"(
 typedef unsigned int u32;
 typedef unsigned long long u64;
 struct ScanParams {
@@ -383,7 +383,9 @@ struct ScanParams {
   u64 n_blocks;             // persistent kernels: blocks of NT * GPT groups in this launch
 };
 static __device__ __forceinline__ u32 fshr(u32 a, u32 b, u32 s) { return __funnelshift_r(a, b, s); }
+)";
 
+const char* kPrelude = R"(
 // One candidate bit (window at bit i of group g, pattern q): an exact re-check by a second method
 // (the window's bases against per-position set masks, mismatches counted by popcount), then the
 // invalid-base test.  Every record is followed by at least one invalid padding base, so a window
@@ -535,14 +537,9 @@ static __device__ __forceinline__ void drain(const ScanParams& P, u64 first, con
 }
 )";
 
-}  // namespace
-
-std::string scan_source(const std::vector<Pattern>& pats, const ScanConfig& cfg, int* alu_ops_per_group) {
+// per-pattern tables of the emission: lengths, budgets, ids, position masks per code and clamp bits
+void emit_pattern_tables(std::ostringstream& os, const std::vector<Pattern>& pats) {
   const int Q = (int)pats.size();
-  std::ostringstream os;
-  os << "// generated scan kernel: " << Q << " patterns\n";
-  os << "#define NT " << cfg.threads << "\n#define GPT " << cfg.groups_per_thread << "\n// shift mode "
-     << cfg.shift_mode << ", persistent " << cfg.persistent << "\n";
   auto table = [&](const char* type, const char* name, auto get) {
     os << "static __device__ const " << type << " " << name << "[" << Q << "] = {";
     for (int q = 0; q < Q; ++q) os << (q ? "," : "") << (unsigned)get(pats[q]);
@@ -570,11 +567,458 @@ std::string scan_source(const std::vector<Pattern>& pats, const ScanConfig& cfg,
     for (int j = p.clamp_lo; j < p.clamp_hi; ++j) m |= 1u << j;
     return m;
   });
+}
+
+// ---- interleaved form -------------------------------------------------------------------------
+// A warp takes 1,024 consecutive groups (32,768 positions) and transposes them: lane l's word i then
+// holds, at bit b, the base at position i of group l + 32 b.  Pattern position j of the windows
+// starting at position i is word i + j of the same lane (past 31: word i + j - 32 of the next
+// group, which is lane l + 1's), so no plane is ever shifted: the transposition costs 16 ALU
+// instructions per 32 positions for both code bits, where the shifted planes cost 46 for the bench
+// pair.  Words are kept one-hot (A, C, T, G) in shared memory; a loop over the 32 positions, IL_R at
+// a time, reads each word once and runs every pattern's filter on it.
+//
+// The filter only has to keep every window that may be a site, since each window it lets through is
+// decided exactly from the bases.  It takes positions free of shifts, so it can afford weak but cheap
+// tests over many of them: the majority of three mismatch bits certifies two mismatches, so
+// ceil(T / 2) such triples certify T (k = 3: five triples and the clamp, 10 instructions with a
+// survival of 4e-5 per window, against 15 for the exact count of nine positions at 1.6e-4).
+// Surviving words go to a queue per warp and the whole warp checks them after its loop.
+//
+// ALU-bound: about 76 ALU instructions per 32 positions for the bench pair (149 in the shifted form),
+// the pipe 86 % busy (ncu).  Against the shifted form: 1.92 Gbp of random bases, bench pair at k = 3
+// 0.290 ms (0.495), four pairs 0.755 (1.353), eight pairs 1.132 (2.551); the 2,000-genome database
+// (7.61 Gbp, k = 3) 1.087 ms (1.808).  Two warps per block and 18.8 KB of shared memory per warp give
+// 12 warps per SM at up to 168 registers; 16-24 warps with the two code planes in place of one-hot
+// words (8.4 KB) ran 6-20 % slower, as did one or three warps per block.  Moving the shifts of the
+// shifted form to the multiply pipe instead (multiplier from constant memory, high or wide products,
+// 15 to 100 % of them) only ran slower: 0.993 to 1.392 ms against 0.980 for 3.84 Gbp.
+
+constexpr int kIlQueue = 96;  // entries of a warp's queue (words of four patterns)
+constexpr int kIlMaxPatterns = 128;
+
+// expected ALU instructions for each surviving word: the push (about 25 by the whole warp) and its
+// share of the queue's check
+constexpr double kIlSurvivor = 35.0;
+
+struct IlPos {
+  uint8_t set;
+  int j;
+  double p_mis;
+};
+
+// the one-hot or derived match plane of set `set` at row `row`, or (inv) its complement; `cache`
+// holds the two-base planes already computed
+Val il_match(Emitter& E, uint8_t set, int row, std::map<std::pair<int, int>, Val>& cache) {
+  const std::string w = "w" + std::to_string(row);
+  auto one = [&](uint8_t s) {
+    return Val{w + (s == SET_A ? ".x" : s == SET_C ? ".y" : s == SET_T ? ".z" : ".w"), false, false};
+  };
+  const int n = __builtin_popcount(set);
+  if (n == 1) return one(set);
+  if (n == 3) {
+    Val v = one((uint8_t)(~set & 15));
+    v.inv = true;
+    return v;
+  }
+  const bool flip = !(set & SET_A);  // the pairs that hold A are computed, the others are complements
+  const uint8_t base = flip ? (uint8_t)(~set & 15) : set;
+  auto it = cache.find({base, row});
+  if (it == cache.end()) {
+    Val v = E.or2(one(SET_A), one((uint8_t)(base & ~SET_A)));
+    it = cache.emplace(std::make_pair((int)base, row), v).first;
+  }
+  Val v = it->second;
+  v.inv = flip;
+  return v;
+}
+
+// A pattern's filter: the clamp and either the first `n` counted positions counted exactly up to T
+// (triples = 0) or the majorities of `triples` triples of them.
+struct IlFilter {
+  std::vector<IlPos> clamp, counted;
+  int T = 1, n = 0, triples = 0;
+  double cost = 0.0, survive = 1.0;
+};
+
+// OR of all terms, three at a time: ceil((n - 1) / 2) instructions
+Val il_or(Emitter& E, std::vector<Val> v) {
+  if (v.empty()) return Val{"", true, true};  // all zeros
+  size_t i = 0;
+  while (v.size() - i >= 3) {
+    v.push_back(E.or3(v[i], v[i + 1], v[i + 2]));
+    i += 3;
+  }
+  return v.size() - i == 2 ? E.or2(v[i], v[i + 1]) : v[i];
+}
+
+// failure word of the filter for the windows at row s
+Val il_emit(Emitter& E, const IlFilter& F, int s, std::map<std::pair<int, int>, Val>& cache) {
+  std::vector<Val> fail;
+  auto mis = [&](const IlPos& p) {
+    Val v = il_match(E, p.set, s + p.j, cache);
+    v.inv = !v.inv;
+    return v;
+  };
+  for (const IlPos& p : F.clamp) fail.push_back(mis(p));
+  std::map<int, std::vector<Val>> bits;
+  int T = F.T;
+  if (F.triples) {
+    for (int t = 0; t < F.triples; ++t)
+      bits[1].push_back(E.maj(mis(F.counted[3 * t]), mis(F.counted[3 * t + 1]), mis(F.counted[3 * t + 2])));
+    T = (F.T + 1) / 2;
+  } else {
+    for (int i = 0; i < F.n; ++i) bits[1].push_back(mis(F.counted[i]));
+  }
+  if ((int)bits[1].size() >= T) {
+    int wsat = 1;
+    while (wsat < T) wsat *= 2;
+    if (wsat == 1) {
+      for (const Val& v : bits[1]) fail.push_back(v);
+    } else {
+      reduce_bits(E, bits, wsat, fail);
+      count_ge(E, bits, wsat, T, fail);
+    }
+  }
+  return il_or(E, fail);
+}
+
+// The filter with the least expected work for windows of uniform random bases, `windows` of them per
+// warp and step: its instructions plus kIlSurvivor for every window it lets through.
+IlFilter il_filter(const Pattern& P, double windows) {
+  IlFilter F;
+  F.T = P.k + 1;
+  for (int j = 0; j < P.len; ++j) {
+    if (P.set[j] == 15) continue;
+    const IlPos p{P.set[j], j, (4 - __builtin_popcount(P.set[j])) / 4.0};
+    (j >= P.clamp_lo && j < P.clamp_hi ? F.clamp : F.counted).push_back(p);
+  }
+  // the positions most likely to mismatch first; among equals one-hot planes before derived ones
+  std::stable_sort(F.counted.begin(), F.counted.end(), [](const IlPos& a, const IlPos& b) { return a.p_mis > b.p_mis; });
+  double p_clamp = 1.0;
+  for (const IlPos& p : F.clamp) p_clamp *= 1.0 - p.p_mis;
+  const int n = (int)F.counted.size();
+  auto fewer = [](const std::vector<double>& ps, int T) {  // P(fewer than T of independent events)
+    std::vector<double> d(T + 1, 0.0);
+    d[0] = 1.0;
+    for (double p : ps) {
+      for (int v = T; v >= 0; --v) d[v] = (v < T ? d[v] * (1.0 - p) : d[v]) + (v ? d[v - 1] * p : 0.0);
+    }
+    return 1.0 - d[T];
+  };
+  bool have = false;
+  IlFilter best;
+  auto consider = [&](int count, int triples) {
+    IlFilter G = F;
+    G.n = count;
+    G.triples = triples;
+    std::vector<double> ps;
+    if (triples) {
+      for (int t = 0; t < triples; ++t) {
+        const double a = F.counted[3 * t].p_mis, b = F.counted[3 * t + 1].p_mis, c = F.counted[3 * t + 2].p_mis;
+        ps.push_back(a * b + a * c + b * c - 2 * a * b * c);
+      }
+    } else {
+      for (int i = 0; i < count; ++i) ps.push_back(F.counted[i].p_mis);
+    }
+    G.survive = p_clamp * fewer(ps, triples ? (F.T + 1) / 2 : F.T);
+    Emitter E;
+    std::map<std::pair<int, int>, Val> cache;
+    il_emit(E, G, 0, cache);
+    G.cost = E.ops + kIlSurvivor * windows * G.survive;
+    if (!have || G.cost < best.cost - 1e-9) best = G, have = true;
+  };
+  for (int c = 0; c <= n; ++c) consider(c, 0);
+  if (F.T >= 2)
+    for (int t = 1; 3 * t <= n; ++t) consider(0, t);
+  return best;
+}
+
+const char* kIlPrelude = R"(
+#define ROW (33 * 16)            // bytes of a row: 32 lanes' words and lane 0's one group on
+#define WARP_GROUPS 1024ull
+
+// 32 x 32 bits: word i bit b = word b bit i of the argument
+static __device__ __forceinline__ void transpose32(u32 (&a)[32]) {
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const u32 x = __byte_perm(a[k], a[k + 16], 0x5410), y = __byte_perm(a[k], a[k + 16], 0x7632);
+    a[k] = x, a[k + 16] = y;
+  }
+#pragma unroll
+  for (int k = 0; k < 32; ++k)
+    if (!(k & 8)) {
+      const u32 x = __byte_perm(a[k], a[k + 8], 0x6240), y = __byte_perm(a[k], a[k + 8], 0x7351);
+      a[k] = x, a[k + 8] = y;
+    }
+#define SWAP_BITS(S, M)                                                                        \
+  _Pragma("unroll") for (int k = 0; k < 32; ++k) if (!(k & S)) {                               \
+    const u32 x = (a[k] & M) | ((a[k + S] << S) & ~M), y = ((a[k] >> S) & M) | (a[k + S] & ~M); \
+    a[k] = x, a[k + S] = y;                                                                    \
+  }
+  SWAP_BITS(4, 0x0f0f0f0fu)
+  SWAP_BITS(2, 0x33333333u)
+  SWAP_BITS(1, 0x55555555u)
+}
+
+// Windows of pattern q at position i of the groups of lane ln (bits of h): decided exactly from the
+// bases against per-position set masks, the mismatches counted by popcount, then the invalid-base
+// test (every record ends in an invalid padding base, so it covers record bounds too), and the
+// sites appended to their tile's slots.  The whole warp takes part, one window per lane and round.
+static __device__ __forceinline__ void check_words(u32 h, int q, u32 i, u32 ln, u64 first, const ScanParams& P) {
+  const u32 lane = threadIdx.x & 31u;
+  while (__any_sync(0xffffffffu, h != 0)) {
+    bool ok = false;
+    u64 key = 0, tile = ~0ull;
+    if (h) {
+      const u32 b = __ffs(h) - 1;
+      h &= h - 1;
+      const u64 gl = first + ln + 32u * b;
+      if (gl < P.n_groups) {
+        const u64 g = P.group_begin + gl;
+        const uint2 x = __ldg(P.planes + g), y = __ldg(P.planes + g + 1);
+        const u64 lo64 = (u64)x.x | ((u64)y.x << 32), hi64 = (u64)x.y | ((u64)y.y << 32);
+        const int L = PLEN[q];
+        const u32 wm = L == 32 ? 0xffffffffu : ((1u << L) - 1u);
+        const u32 wl = (u32)(lo64 >> i), wh = (u32)(hi64 >> i);  // base j of the window at bit j
+        const u32 match = (~wl & ~wh & MSET[q][0]) | (wl & ~wh & MSET[q][1]) | (~wl & wh & MSET[q][2]) |
+                          (wl & wh & MSET[q][3]);
+        const u32 mis = ~match & wm;
+        const int mism = __popc(mis);
+        if (!(mis & PCLAMP[q]) && mism <= PK[q]) {
+          const u64 inv64 = (u64)P.invalid[g] | ((u64)P.invalid[g + 1] << 32);
+          if (!((u32)(inv64 >> i) & wm)) {
+            const u64 pos = g * 32ull + (u64)i;
+            tile = g / P.tile_groups;
+            key = ((u64)PPAIR[q] << 48) | ((pos - tile * P.tile_groups * 32ull) << 16) | ((u64)PORIENT[q] << 8) |
+                  (u64)mism;
+            ok = true;
+          }
+        }
+      }
+    }
+    // the lanes of one tile take their slots with one atomic add
+    const u32 peers = __match_any_sync(0xffffffffu, tile);
+    if (ok) {
+      const u32 leader = __ffs(peers) - 1;
+      u32 base = 0;
+      if (lane == leader) base = atomicAdd(P.tile_count + tile, (u32)__popc(peers));
+      base = __shfl_sync(peers, base, leader);
+      const u32 idx = base + __popc(peers & ((1u << lane) - 1u));
+      if (idx < P.slot_cap) P.slots[tile * (u64)P.slot_cap + idx] = key;
+    }
+  }
+}
+
+// the queue's first n entries of positions below i_end, an entry per lane, its words one after
+// another (mostly it holds one)
+static __device__ __noinline__ void drain(u32 n, u32 i_end, u64 first, const ScanParams& P, const uint4* qw,
+                                          const u32* qm) {
+  for (u32 e0 = 0; e0 < n; e0 += 32) {
+    const u32 e = e0 + (threadIdx.x & 31u);
+    const u32 m = e < n ? qm[e] : 0u;
+    const uint4 c = e < n && ((m >> 16) & 31u) < i_end ? qw[e] : make_uint4(0u, 0u, 0u, 0u);
+    u32 left = (c.x ? 1u : 0u) | (c.y ? 2u : 0u) | (c.z ? 4u : 0u) | (c.w ? 8u : 0u);
+    while (__any_sync(0xffffffffu, left != 0)) {
+      const int t = left ? __ffs(left) - 1 : 0;
+      const u32 h = left == 0 ? 0u : t == 0 ? c.x : t == 1 ? c.y : t == 2 ? c.z : c.w;
+      left &= left - 1;
+      check_words(h, (int)(m & 0xffffu) + t, (m >> 16) & 31u, m >> 24, first, P);
+    }
+  }
+}
+
+// A warp's queue of surviving words: an entry holds a lane's words of a block of four patterns at one
+// position.
+struct Queue {
+  uint4 w[QCAP];
+  u32 m[QCAP];  // first pattern | position << 16 | lane << 24
+  u32 n;        // entries asked for
+};
+
+// A lane's surviving windows of patterns q0 .. q0+3 at position i into its warp's queue: counted, but
+// dropped when it is full (the tile or iteration is then run again).  By the lanes that hold a word,
+// with an atomic add: a vote of the whole warp and the count in a register ran 6 % slower, since
+// each vote keeps the instructions around it in order.
+static __device__ __forceinline__ void push4(u32 c0, u32 c1, u32 c2, u32 c3, int q0, u32 i, Queue& Q) {
+  const u32 idx = atomicAdd(&Q.n, 1u);
+  if (idx < QCAP) {
+    Q.w[idx] = make_uint4(c0, c1, c2, c3);
+    Q.m[idx] = (u32)q0 | (i << 16) | ((threadIdx.x & 31u) << 24);
+  }
+}
+)";
+
+// Positions per loop iteration: more read each row fewer times, until the rows in use overflow the
+// registers and the loop body the instruction cache.  1.92 Gbp of random bases, 8 / 4 / 2 positions:
+// one pair 0.290 / 0.320 ms, two pairs 0.440 / 0.460, four pairs 0.802 / 0.755 / 0.852, eight pairs
+// 1.480 / 1.132 / 1.228.
+int il_rows(int patterns) { return patterns <= 8 ? 8 : patterns <= 32 ? 4 : 2; }
+// Blocks per SM the registers must allow (shared memory holds six): at six the compiler takes up to 168
+// registers; one pair needs fewer and ran 4 % faster bounded for seven.
+int il_blocks(int patterns) { return patterns <= 4 ? 7 : 6; }
+
+std::string interleaved_source(const std::vector<Pattern>& pats, const ScanConfig& cfg, int* alu_ops_per_group) {
+  const int Q = (int)pats.size(), R = cfg.il_rows > 0 ? cfg.il_rows : il_rows(Q);
+  std::ostringstream os;
+  os << "// generated scan kernel, interleaved form: " << Q << " patterns\n";
+  os << "#define NT " << 32 * kIlWarps << "\n#define QCAP " << kIlQueue << "\n";
+  emit_pattern_tables(os, pats);
+  os << kParams << kIlPrelude;
+  // the loop body: R positions of every pattern
+  std::vector<IlFilter> filt;
+  for (const Pattern& P : pats) filt.push_back(il_filter(P, std::max(1, cfg.vote_windows)));
+  Emitter E;
+  std::map<std::pair<int, int>, Val> cache;
+  for (int s = 0; s < R; ++s) {
+    // rows are read as they come into use: with every read hoisted to the loop's start the registers
+    // overflowed and larger sets ran 5-25 % slower
+    if (s) E.os << "    asm volatile(\"\" ::: \"memory\");\n@ROW" << s << "\n";
+    for (int q0 = 0; q0 < Q; q0 += 4) {
+      const int q1 = std::min(Q, q0 + 4);
+      std::string f[4];
+      for (int q = q0; q < q1; ++q) {
+        f[q - q0] = "f" + std::to_string(q) + "_" + std::to_string(s);
+        const Val v = il_emit(E, filt[q], s, cache);
+        E.os << "    const u32 " << f[q - q0] << " = " << expr_of(v) << ";\n";
+      }
+      E.os << "    if (__builtin_expect((";
+      for (int q = q0; q < q1; ++q) E.os << (q > q0 ? " & " : "") << f[q - q0];
+      E.os << ") != 0xffffffffu && on, 0)) push4(";
+      for (int t = 0; t < 4; ++t) E.os << (q0 + t < q1 ? "~" + f[t] : std::string("0u")) << ", ";
+      E.os << q0 << ", i0 + " << s << "u, qu);\n";
+    }
+  }
+  std::string body = E.os.str();
+  int rows = R;  // rows the filters read
+  for (const IlFilter& F : filt) {
+    for (const IlPos& p : F.clamp) rows = std::max(rows, R + p.j);
+    for (int i = 0; i < (F.triples ? 3 * F.triples : F.n); ++i) rows = std::max(rows, R + F.counted[i].j);
+  }
+  // per 32 positions: transposition and one-hot planes (20), the filters, a test per block of four
+  if (alu_ops_per_group) *alu_ops_per_group = 20 + (E.ops + R - 1) / R + 3 * ((Q + 3) / 4);
+  os << "extern \"C\" __global__ void __launch_bounds__(NT, " << (cfg.min_blocks > 0 ? cfg.min_blocks : il_blocks(Q))
+     << ") ah_scan_jit(const __grid_constant__ ScanParams P) {\n";
+  os << R"(  __shared__ __align__(16) unsigned char rows_sm[NT / 32][32 * ROW];
+  __shared__ Queue queue[NT / 32];
+  const u32 lane = threadIdx.x & 31u, wp = threadIdx.x >> 5;
+  unsigned char* V = rows_sm[wp];
+  Queue& qu = queue[wp];
+  const u64 first = ((u64)blockIdx.x * (NT / 32) + wp) * WARP_GROUPS;
+  if (first >= P.n_groups) return;
+  if (lane == 0) qu.n = 0;
+  // tiles that a later block will read, into L2 (2 % on the bench pair; 456 to 2,736 tiles ahead alike)
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const u64 gl = first + 912ull * WARP_GROUPS + (u64)(lane * 16u + k * 512u);
+    if (gl < P.n_groups) asm volatile("prefetch.global.L2 [%0];" ::"l"(P.planes + P.group_begin + gl));
+  }
+  {
+    // bit b of a lane's words: group first + lane + 32 b; the group after the last one is read too
+    // (windows of the last group run into it), later ones stand as A and are refused when checked
+    u32 lo[32], hi[32];
+#pragma unroll
+    for (int b = 0; b < 32; ++b) {
+      const u64 gl = first + lane + 32 * b;
+      uint2 v = make_uint2(0u, 0u);
+      if (gl <= P.n_groups) v = __ldg(P.planes + P.group_begin + gl);
+      lo[b] = v.x, hi[b] = v.y;
+    }
+    transpose32(lo);
+    transpose32(hi);
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      *(uint4*)(V + i * ROW + lane * 16) = make_uint4(~(lo[i] | hi[i]), lo[i] & ~hi[i], ~lo[i] & hi[i], lo[i] & hi[i]);
+  }
+  __syncwarp();
+  {
+    // column 32 is lane 0's words one group on: shifted down by a bit, the group after the tile on top
+    const u64 gn = first + WARP_GROUPS;
+    uint2 v = make_uint2(0u, 0u);
+    if (gn <= P.n_groups) v = __ldg(P.planes + P.group_begin + gn);
+    const u32 l = (v.x >> lane) & 1u, h = (v.y >> lane) & 1u;
+    uint4 x = *(const uint4*)(V + lane * ROW);
+    x.x = (x.x >> 1) | ((1u ^ (l | h)) << 31);
+    x.y = (x.y >> 1) | ((l & ~h) << 31);
+    x.z = (x.z >> 1) | ((~l & h & 1u) << 31);
+    x.w = (x.w >> 1) | ((l & h) << 31);
+    *(uint4*)(V + lane * ROW + 512) = x;
+  }
+  __syncwarp();
+  const unsigned char* L0 = V + lane * 16;
+#pragma unroll 1
+)";
+  // The queue is checked after the loop; when it overflowed the tile is run again with care: the queue
+  // checked after every iteration, and an iteration that overflows it run again for a few lanes at a
+  // time (the others muted), so few that the queue holds all they may find.  Sets whose survivors
+  // would often fill the queue start with care.
+  const int lanes = kIlQueue / (R * ((Q + 3) / 4));
+  double expect = 0.0;
+  for (const IlFilter& F : filt) expect += 32768.0 * F.survive;
+  os << "  bool on = true;\n  u32 sel = ~0u;  // sel: first lane of an iteration run again, ~0 otherwise\n";
+  os << "  bool care = " << (expect > kIlQueue / 4 ? "true" : "false") << ";\n";
+  os << "  for (u32 i0 = 0;;) {\n";
+  os << R"(    if (i0 == 32u) {
+      __syncwarp();
+      if (care || qu.n <= QCAP) break;
+      __syncwarp();
+      if (lane == 0) qu.n = 0;
+      __syncwarp();
+      care = true;
+      i0 = 0;
+    }
+)";
+  for (int q = 0; q * R < rows; ++q)
+    os << "    const unsigned char* B" << q << " = L0 + ((i0 + " << q * R << "u) & 31u) * ROW + ((i0 + " << q * R
+       << "u) >> 5) * 16;\n";
+  for (int r = 0; r < rows; ++r) {
+    const std::string load = "    const uint4 w" + std::to_string(r) + " = *(const uint4*)(B" + std::to_string(r / R) +
+                             " + " + std::to_string(r % R) + " * ROW);\n";
+    const int s = r - (rows - R);  // the first position that reads the row
+    if (s <= 0) {
+      os << load;
+      continue;
+    }
+    const std::string mark = "@ROW" + std::to_string(s) + "\n";
+    body.replace(body.find(mark), mark.size(), load);
+  }
+  os << body;
+  os << "    if (!care) {\n      i0 += " << R << ";\n      continue;\n    }\n";
+  os << "    __syncwarp();\n    const u32 n = qu.n;\n";
+  os << "    if (sel == ~0u && n <= QCAP / 2) {\n      i0 += " << R << ";\n      continue;\n    }\n";
+  os << "    const bool again = sel == ~0u && n > QCAP;\n";
+  os << "    drain(min(n, (u32)QCAP), again ? i0 : 32u, first, P, qu.w, qu.m);\n    __syncwarp();\n";
+  os << "    if (lane == 0) qu.n = 0;\n    __syncwarp();\n";
+  os << "    sel = again ? 0u : sel == ~0u || sel + " << lanes << "u >= 32u ? ~0u : sel + " << lanes << "u;\n";
+  os << "    on = sel == ~0u || lane - sel < " << lanes << "u;\n";
+  os << "    if (sel == ~0u) i0 += " << R << ";\n  }\n";
+  os << "  drain(qu.n, 32u, first, P, qu.w, qu.m);\n}\n";
+  return os.str();
+}
+
+}  // namespace
+
+bool interleaved_suits(const std::vector<Pattern>& pats) {
+  const int Q = (int)pats.size();
+  if (Q == 0 || Q > kIlMaxPatterns) return false;
+  double per_iteration = 0.0;
+  for (const Pattern& P : pats) per_iteration += il_rows(Q) * 1024.0 * il_filter(P, 1024.0).survive;
+  return per_iteration <= kIlQueue / 2;
+}
+
+std::string scan_source(const std::vector<Pattern>& pats, const ScanConfig& cfg, int* alu_ops_per_group) {
+  if (cfg.interleaved) return interleaved_source(pats, cfg, alu_ops_per_group);
+  const int Q = (int)pats.size();
+  std::ostringstream os;
+  os << "// generated scan kernel: " << Q << " patterns\n";
+  os << "#define NT " << cfg.threads << "\n#define GPT " << cfg.groups_per_thread << "\n// shift mode "
+     << cfg.shift_mode << ", persistent " << cfg.persistent << "\n";
+  emit_pattern_tables(os, pats);
   // direct emission: the routine inlined at up to two call sites (8 patterns; measured on GB300 the
   // dense-site workload, 4 patterns, scanned 5 % faster inlined and the 32-pattern set 5 % slower);
   // with the queue it is only the rare fallback
   os << "#define EMIT_INLINE " << (!cfg.emit_queue && Q <= 8 ? "__forceinline__" : "__noinline__") << "\n";
-  os << kPrelude;
+  os << kParams << kPrelude;
 
   // body: per group of 32 positions
   Emitter E;
@@ -763,8 +1207,9 @@ ah_status load(int device, const std::vector<char>& cubin, int ops, const ScanCo
     *err = std::string("cudaLibraryGetKernel failed: ") + cudaGetErrorString(ce);
     return AH_EJIT;
   }
-  k->threads = cfg.threads;
-  k->groups_per_thread = cfg.groups_per_thread;
+  k->threads = cfg.interleaved ? 32 * kIlWarps : cfg.threads;
+  k->tile_groups = scan_tile_groups(cfg);
+  k->block_groups = scan_block_groups(cfg);
   k->alu_ops_per_group = ops;
   return AH_OK;
 }

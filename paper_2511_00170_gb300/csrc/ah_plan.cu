@@ -291,6 +291,13 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
   pl->prm = *prm;
   pl->cfg = ctx->scan_cfg;
   pl->cfg.pairs_per_kernel = 0;  // a plan captures one scan kernel over every pair
+  // Plans scan in the interleaved form where it suits the primers: 1.6x (one pair) to 2.2x (eight) as
+  // fast, for a compile of 0.45 s instead of 0.16 s (one pair; 1 s instead of 0.45 s for eight), which
+  // a plan's replays repay and a single scan of a new primer set would not.  Few tiles keep the shifted
+  // form: a tile is one warp's work for 13 us (one pair) to 25 us (eight), the shifted form's 10 to
+  // 20; they meet at 16 Mbp (one pair), 10 (four) and 8 (eight), and 512 tiles are 16.8 Mbp.
+  pl->cfg.interleaved = !ctx->scan_cfg_given && prm->persistent <= 0 && b->n_groups >= 512ull * kIlTileGroups &&
+                        interleaved_suits(p->pats);
   ah_status st = tm_prepare(ctx, &prm->tm, pl->tm_run, sizeof pl->tm_run);
   if (!st && !prm->tm.variants) st = tm_kernel_for(ctx, p, true, tm_run_slot(pl->tm_run), &pl->tm_k);
   for (int i = 0; i < 2 && !st; ++i)
@@ -300,12 +307,23 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
   if (!st && prm->autotune) {
     // candidate shapes x alignment modes, then the persistent form of the best; a candidate replaces
     // the incumbent only when it is at least 3 % faster, so near-equal shapes do not flip between runs
-    const int shapes[][2] = {{256, 8}, {128, 8}, {256, 4}, {128, 4}};
+    const int shapes[][2] = {{128, 8}, {256, 8}, {256, 4}, {128, 4}};
     double best = 1e30;
     ScanConfig win = pl->cfg;
-    for (int mode = 0; mode < 2 && !st; ++mode) {
+    // the interleaved form first; where it beats the shifted form's first shape by a tenth (1.7x on the
+    // bench pair) the other shifted candidates, within a few percent of each other, are not tried
+    bool shifted = true;
+    if (win.interleaved) {
+      ScanConfig c = win;
+      c.interleaved = 0;
+      double ms = 0;
+      if (!(st = time_shape(ctx, b, p, win, 2, &best, &n_hits))) st = time_shape(ctx, b, p, c, 2, &ms, &n_hits);
+      shifted = ms < best * 1.1;
+    }
+    for (int mode = 0; mode < 2 && !st && shifted; ++mode) {
       for (auto& sh : shapes) {
         ScanConfig c = pl->cfg;
+        c.interleaved = 0;
         c.threads = sh[0];
         c.groups_per_thread = sh[1];
         c.shift_mode = mode;
@@ -317,7 +335,7 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
     }
     // a large circuit (the 8-pair batched set: 166 registers, 3 blocks of 128 threads per SM) may
     // run faster with registers bounded for 4 blocks: more warps, a few spills to L1
-    if (!st && win.threads == 128 && ctx->scan_ops_per_group > 400) {
+    if (!st && !win.interleaved && win.threads == 128 && ctx->scan_ops_per_group > 400) {
       ScanConfig c = win;
       c.min_blocks = 4;
       double ms = 0;
@@ -335,13 +353,13 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
     // candidates queued per warp and emitted by the whole warp after its block: pays where sites are
     // dense (tandem repeats: the dense workload's scan went from 8.6 to 6.2 ms), costs a little
     // elsewhere (registers and shared memory)
-    if (!st) {
+    if (!st && !win.interleaved) {
       ScanConfig c = win;
       c.emit_queue = 1;
       double ms = 0;
       if (!(st = time_shape(ctx, b, p, c, 2, &ms, &n_hits)) && ms < best * 0.97) best = ms, win = c;
     }
-    if (!st && prm->persistent != 0) {
+    if (!st && !win.interleaved && prm->persistent != 0) {
       ScanConfig c = win;
       c.persistent = 1;
       double ms = 0;
@@ -375,7 +393,7 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
   ah_amplicons_free(a);
   if (!st) st = ctx->jit->get(ctx, p->pats, pl->cfg, &pl->kern);
   if (!st) {
-    pl->tile_groups = (uint64_t)pl->cfg.threads * pl->cfg.groups_per_thread;
+    pl->tile_groups = pl->kern.tile_groups;
     pl->n_tiles = std::max<uint64_t>(1, (b->n_groups + pl->tile_groups - 1) / pl->tile_groups);
     pl->n_cells = (uint64_t)p->n_pairs * pl->n_tiles;
     pl->slot_cap = (uint32_t)pl->cfg.slot_cap;
@@ -412,14 +430,15 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
     ah_plan_free(pl);
     return st;
   }
-  pl->info.threads = pl->cfg.threads;
-  pl->info.groups_per_thread = pl->cfg.groups_per_thread;
+  pl->info.threads = pl->kern.threads;
+  pl->info.groups_per_thread = (int32_t)(pl->kern.block_groups / pl->kern.threads);
   pl->info.shift_mode = pl->cfg.shift_mode;
   pl->info.persistent = pl->cfg.persistent;
   pl->info.min_blocks = pl->cfg.min_blocks;
   pl->info.vote_windows = pl->cfg.vote_windows;
   pl->info.emit_queue = pl->cfg.emit_queue;
-  pl->info.grid = pl->grid ? pl->grid : (int32_t)pl->n_tiles;
+  pl->info.grid = pl->grid ? pl->grid
+                             : (int32_t)((pl->n_tiles * pl->tile_groups + pl->kern.block_groups - 1) / pl->kern.block_groups);
   *out = pl;
   return AH_OK;
 }
@@ -497,7 +516,7 @@ ah_status ah_plan_launch_host(ah_plan* pl, const uint8_t* h_seq, const uint64_t*
   enqueue_pre(pl, c->stream);
   // tiles whose groups and the group after them are packed are scanned at once, while the next
   // chunk crosses the link
-  const uint64_t tg = (uint64_t)pl->range_kern.threads * pl->range_kern.groups_per_thread;
+  const uint64_t tg = pl->range_kern.tile_groups;
   uint64_t scanned = 0;
   uint64_t scan_launches = 0;
   auto on_chunk = [&](uint64_t done) {
@@ -560,7 +579,7 @@ ah_status ah_plan_launch_packed(ah_plan* pl, const void* h_planes, uint64_t n_in
   if (e == cudaSuccess) e = cudaEventRecord(ready, c->stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ready, 0);
   if (e == cudaSuccess && (st = scatter_invalid_list(c, b, &il))) e = cudaErrorUnknown;
-  const uint64_t tg = (uint64_t)pl->range_kern.threads * pl->range_kern.groups_per_thread;
+  const uint64_t tg = pl->range_kern.tile_groups;
   uint64_t scanned = 0, scan_launches = 0;
   for (uint64_t k = 0; k < n_chunks && e == cudaSuccess; ++k) {
     const uint64_t g0 = k * chunk, g1 = std::min(b->n_groups, g0 + chunk);
@@ -614,7 +633,7 @@ ah_status ah_plan_launch_fasta(ah_plan* pl, const char* text, uint64_t n_bytes) 
   std::vector<uint64_t> start(b->n_records + 1, 0);
   for (uint32_t r = 0; r < b->n_records; ++r) start[r + 1] = start[r] + b->h_rec_len[r];
   ConcatCursor cur;
-  const uint64_t tg = (uint64_t)pl->range_kern.threads * pl->range_kern.groups_per_thread;
+  const uint64_t tg = pl->range_kern.tile_groups;
   uint64_t scanned = 0, scan_launches = 0;
   // after each chunk: pack the record bases it completed, then scan the tiles whose groups (and the
   // group after them) are packed, while the next chunk of text crosses the link

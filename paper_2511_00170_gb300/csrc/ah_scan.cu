@@ -447,22 +447,22 @@ std::vector<GenPattern> gen_table(const std::vector<Pattern>& pats) {
 
 void launch_scan_kernel(cudaStream_t s, const ScanKernel& k, const ah_batch* b, uint64_t* slots, uint32_t* tile_count,
                         uint32_t cap, uint32_t* status, unsigned long long* work, uint64_t n_tiles, int grid) {
-  // whole batch, tiles of threads * groups_per_thread groups; grid > 0 selects the persistent form
-  const uint64_t tg = (uint64_t)k.threads * k.groups_per_thread;
+  // the whole batch; grid > 0 selects the persistent form (whose blocks are tiles)
+  const uint64_t tg = k.tile_groups, n_blocks = (n_tiles * tg + k.block_groups - 1) / k.block_groups;
   ScanParamsHost P{b->planes, b->invalid, b->rec_group, b->rec_len, b->n_records, cap, 0, b->n_groups,
                    slots, tile_count, status, tg, work, n_tiles};
   void* args[] = {&P};
-  cudaLaunchKernel((const void*)k.fn, dim3((unsigned)(grid > 0 ? grid : n_tiles)), dim3((unsigned)k.threads), args, 0, s);
+  cudaLaunchKernel((const void*)k.fn, dim3((unsigned)(grid > 0 ? grid : n_blocks)), dim3((unsigned)k.threads), args, 0, s);
 }
 
 void launch_scan_range(cudaStream_t s, const ScanKernel& k, const ah_batch* b, uint64_t* slots, uint32_t* tile_count,
                        uint32_t cap, uint32_t* status, uint64_t g0, uint64_t g1) {
-  const uint64_t tg = (uint64_t)k.threads * k.groups_per_thread;
+  const uint64_t tg = k.tile_groups, bg = k.block_groups;
   if (g1 <= g0) return;
   ScanParamsHost P{b->planes, b->invalid, b->rec_group, b->rec_len, b->n_records, cap, g0, g1 - g0,
                    slots, tile_count, status, tg, nullptr, 0};
   void* args[] = {&P};
-  cudaLaunchKernel((const void*)k.fn, dim3((unsigned)((g1 - g0 + tg - 1) / tg)), dim3((unsigned)k.threads), args, 0, s);
+  cudaLaunchKernel((const void*)k.fn, dim3((unsigned)((g1 - g0 + bg - 1) / bg)), dim3((unsigned)k.threads), args, 0, s);
 }
 
 void launch_tile_max(cudaStream_t s, const uint32_t* tile_count, uint64_t n_tiles, uint32_t* out) {
@@ -565,9 +565,10 @@ ah_status enqueue_jit(ah_ctx* ctx, const ah_batch* b, const std::vector<ScanKern
                        std::min<uint64_t>(b->n_groups - std::min(b->n_groups, g0), nt * tile_groups),
                        slots, tile_count, ctx->d_status, tile_groups, work, nt};
       void* args[] = {&P};
-      const unsigned grid =
-          cfg.persistent ? (unsigned)std::min<uint64_t>(nt, persistent_grid(ctx, kern)) : (unsigned)nt;
-      cudaError_t le = cudaLaunchKernel((const void*)kern.fn, dim3(grid), dim3((unsigned)cfg.threads), args, 0,
+      const unsigned grid = cfg.persistent
+                                ? (unsigned)std::min<uint64_t>(nt, persistent_grid(ctx, kern))
+                                : (unsigned)((nt * tile_groups + kern.block_groups - 1) / kern.block_groups);
+      cudaError_t le = cudaLaunchKernel((const void*)kern.fn, dim3(grid), dim3((unsigned)kern.threads), args, 0,
                                         ctx->stream);
       if (le != cudaSuccess) return fail(ctx, AH_ECUDA, "scan kernel launch failed: %s", cudaGetErrorString(le));
       launched(ctx);
@@ -658,7 +659,6 @@ ah_status launch_scan(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const
     return AH_OK;
   }
   // one launch per record per pair, each with the pair's four oriented patterns
-  const uint64_t blk_groups = (uint64_t)cfg.threads * cfg.groups_per_thread;
   if (ctx->timing) AH_CUDA(ctx, cudaEventRecord(ctx->ev[0], ctx->stream));
   for (uint32_t pair = 0; pair < p->n_pairs; ++pair) {
     std::vector<Pattern> pats(p->pats.begin() + 4 * pair, p->pats.begin() + 4 * pair + 4);
@@ -670,8 +670,8 @@ ah_status launch_scan(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const
       ScanParamsHost P{b->planes, b->invalid, b->rec_group, b->rec_len, b->n_records, cap, g0, ng,
                        slots, tile_count, ctx->d_status, tile_groups, nullptr, 0};
       void* args[] = {&P};
-      cudaError_t le = cudaLaunchKernel((const void*)kern.fn, dim3((unsigned)((ng + blk_groups - 1) / blk_groups)),
-                                        dim3((unsigned)cfg.threads), args, 0, ctx->stream);
+      cudaError_t le = cudaLaunchKernel((const void*)kern.fn, dim3((unsigned)((ng + kern.block_groups - 1) / kern.block_groups)),
+                                        dim3((unsigned)kern.threads), args, 0, ctx->stream);
       if (le != cudaSuccess) return fail(ctx, AH_ECUDA, "scan kernel launch failed: %s", cudaGetErrorString(le));
       launched(ctx);
       ctx->n_scan_launches++;
@@ -695,7 +695,7 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
   uint64_t n_tiles = 0, tile_groups = 0;
   uint32_t cap = (uint32_t)cfg.slot_cap;
   for (;;) {
-    tile_groups = (uint64_t)cfg.threads * cfg.groups_per_thread;
+    tile_groups = scan_tile_groups(cfg);
     n_tiles = std::max<uint64_t>(1, (b->n_groups + tile_groups - 1) / tile_groups);
     if ((st = dalloc(ctx, &slots, n_tiles * cap))) break;
     if ((st = dalloc(ctx, &tile_count, n_tiles))) break;
@@ -725,6 +725,7 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
       cap = need;
     } else {
       cap = 4096;
+      if (cfg.interleaved) cfg.interleaved = 0;  // its tiles do not shrink
       if (cfg.groups_per_thread > 1) cfg.groups_per_thread = 1;
       else if (cfg.threads > 64) cfg.threads /= 2;
       else return fail(ctx, AH_EOVERFLOW, "scan: more than %u sites in a tile of %d groups", mx, cfg.threads);

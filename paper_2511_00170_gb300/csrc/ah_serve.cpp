@@ -321,7 +321,7 @@ ah_status ah_server_submit(ah_server* s, const ah_request* r, uint64_t* ticket) 
   j->req.fwd = j->req.rev = nullptr;
   j->req.k = nullptr;
   j->result = (ah_result*)calloc(1, sizeof(ah_result));
-  j->est_bytes = estimate_bytes(s, *r, 64, (uint64_t)s->ctxs[0]->scan_cfg.threads * s->ctxs[0]->scan_cfg.groups_per_thread);
+  j->est_bytes = estimate_bytes(s, *r, 64, scan_tile_groups(s->ctxs[0]->scan_cfg));
   j->reserved = j->est_bytes;
   {
     std::lock_guard<std::mutex> lock(s->mu);
@@ -381,7 +381,7 @@ ah_status ah_server_inject_alloc_failures(ah_server* s, int n) {
 ah_status ah_server_request_bytes(const ah_server* s, const ah_request* r, uint64_t* bytes) {
   if (!s || !r || !bytes || r->n_records == 0 || (uint64_t)r->first_record + r->n_records > s->db->n_records)
     return AH_EINVAL;
-  *bytes = estimate_bytes(s, *r, 64, (uint64_t)s->ctxs[0]->scan_cfg.threads * s->ctxs[0]->scan_cfg.groups_per_thread);
+  *bytes = estimate_bytes(s, *r, 64, scan_tile_groups(s->ctxs[0]->scan_cfg));
   return AH_OK;
 }
 
