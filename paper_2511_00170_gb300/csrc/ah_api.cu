@@ -437,6 +437,7 @@ ah_status ah_ctx_create(ah_ctx** out, int device, void* cuda_stream) {
   }
   if (cudaMalloc(&ctx->d_status, sizeof(uint32_t)) != cudaSuccess ||
       cudaMallocHost(&ctx->h_status, sizeof(uint32_t)) != cudaSuccess ||
+      cudaMallocHost(&ctx->h_read, kReadWords * sizeof(uint64_t)) != cudaSuccess ||
       cudaMemset(ctx->d_status, 0, sizeof(uint32_t)) != cudaSuccess) {
     ah_ctx_destroy(ctx);
     return AH_ENOMEM;
@@ -477,6 +478,7 @@ void ah_ctx_destroy(ah_ctx* ctx) {
   }
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->h_status) cudaFreeHost(ctx->h_status);
+  if (ctx->h_read) cudaFreeHost(ctx->h_read);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
 }
@@ -485,9 +487,8 @@ const char* ah_last_error(const ah_ctx* ctx) { return ctx ? ctx->err.c_str() : "
 
 ah_status ah_ctx_synchronize(ah_ctx* ctx) {
   if (!ctx) return AH_EINVAL;
-  AH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   ah_status st = drain_timings(ctx);
-  return st ? st : check_status(ctx);
+  return st ? st : check_status(ctx);  // synchronises
 }
 
 void* ah_ctx_stream(const ah_ctx* ctx) { return ctx ? (void*)ctx->stream : nullptr; }

@@ -549,6 +549,9 @@ ah_status fasta_pack(ah_ctx* ctx, const char* text, uint64_t n_bytes, const uint
                     (void*)tile_hdr, (void*)seq_base, (void*)hdr_base, (void*)hdr_pos, (void*)hdr_end, (void*)seq_rank})
       dfree(ctx, p);
   };
+  auto read_totals = [&](std::vector<const uint64_t*> d, std::vector<uint64_t*> h) {
+    return read_u64s(ctx, (int)d.size(), d.data(), h.data());
+  };
   // record arrays with room for `need` records, contents kept, a missing header end read as the end
   // of the text
   auto grow = [&](uint64_t need) -> ah_status {
@@ -630,7 +633,7 @@ ah_status fasta_pack(ah_ctx* ctx, const char* text, uint64_t n_bytes, const uint
       uint64_t c_seq = 0, c_hdr = 0;
       if ((st = exclusive_scan_u32(ctx, tile_seq + t0, seq_base + t0, nt)) ||
           (st = exclusive_scan_u32(ctx, tile_hdr + t0, hdr_base + t0, nt)) ||
-          (st = read_u64(ctx, seq_base + t0 + nt, &c_seq)) || (st = read_u64(ctx, hdr_base + t0 + nt, &c_hdr)))
+          (st = read_totals({seq_base + t0 + nt, hdr_base + t0 + nt}, {&c_seq, &c_hdr})))
         break;
       if (c_hdr && (st = grow(total_hdr + c_hdr))) break;
       // pass 3: the chunk's bases and headers at their places in the whole text
@@ -785,6 +788,9 @@ ah_status ah_fastq_pack(ah_ctx* ctx, const char* text, uint64_t n_bytes, const u
     k_fill_u64<<<(unsigned)std::min<uint64_t>((n + 255) / 256, 4096), 256, 0, ctx->stream>>>(p, n, v);
     launched(ctx);
   };
+  auto read_totals = [&](std::vector<const uint64_t*> d, std::vector<uint64_t*> h) {
+    return read_u64s(ctx, (int)d.size(), d.data(), h.data());
+  };
   // record arrays with room for `need` records, contents kept; a new record's header end reads as
   // the end of the text and its rank as missing (~0) until its header is seen
   auto grow = [&](uint64_t need) -> ah_status {
@@ -873,8 +879,8 @@ ah_status ah_fastq_pack(ah_ctx* ctx, const char* text, uint64_t n_bytes, const u
       if ((st = exclusive_scan_u32(ctx, tile_seq + t0, seq_base + t0, nt)) ||
           (st = exclusive_scan_u32(ctx, tile_qual + t0, qual_base + t0, nt)) ||
           (st = exclusive_scan_u32(ctx, tile_hdr + t0, hdr_base + t0, nt)) ||
-          (st = read_u64(ctx, line_base + t0 + nt, &c_lines)) || (st = read_u64(ctx, seq_base + t0 + nt, &c_seq)) ||
-          (st = read_u64(ctx, qual_base + t0 + nt, &c_qual)) || (st = read_u64(ctx, hdr_base + t0 + nt, &c_hdr)))
+          (st = read_totals({line_base + t0 + nt, seq_base + t0 + nt, qual_base + t0 + nt, hdr_base + t0 + nt},
+                            {&c_lines, &c_seq, &c_qual, &c_hdr})))
         break;
       if ((st = grow(n_rec + c_hdr)) || (st = grow_bytes(&seq, &seq_cap, total_seq, total_seq + c_seq)) ||
           (st = grow_bytes(&qual, &qual_cap, total_qual, total_qual + c_qual)))

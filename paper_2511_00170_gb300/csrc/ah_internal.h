@@ -120,6 +120,7 @@ struct ah_ctx {
   cudaEvent_t bounce_ev[2] = {nullptr, nullptr};
   uint32_t* d_status = nullptr;      // device status word
   uint32_t* h_status = nullptr;      // pinned mirror
+  uint64_t* h_read = nullptr;        // page-locked words for counts read back (kReadWords)
   ah::JitCache* jit = nullptr;       // the process-wide kernel cache
   std::mutex stats_mu;               // compile counters are updated from compile threads
   ah::ScanConfig scan_cfg;
@@ -252,8 +253,11 @@ ah_status exclusive_scan_u64(ah_ctx* ctx, const uint64_t* d_in, uint64_t* d_out,
 // pageable path (one staging pipeline for every stream of the process)
 ah_status copy_to_host(ah_ctx* ctx, void* dst, const void* src, uint64_t bytes);
 constexpr uint64_t kBounceBytes = 8ull << 20;  // each of a context's two bounce buffers
-// read one uint64 from device memory (synchronises the stream)
+constexpr int kReadWords = 512;  // page-locked words of a context for counts read back
+// read one uint64 (or n of them, at most 8, from places of their own) from device memory through the
+// context's page-locked words, in one synchronisation of the stream
 ah_status read_u64(ah_ctx* ctx, const uint64_t* d, uint64_t* h);
+ah_status read_u64s(ah_ctx* ctx, int n, const uint64_t* const* d, uint64_t* const* h);
 // A batch of n records whose bases lie in device memory at d_seq[rank[r], rank[r + 1]) (rank[n] =
 // total), with the ranks both on the device (d_rank, n values) and on the host (h_rank, n + 1
 // values).  Lengths, group offsets and packing items are computed on the device; the batch's host
@@ -400,7 +404,7 @@ ah_status nvrtc_compile(int device, const std::string& src, const char* name, st
 // the same for compute capability sm (e.g. 103), with no device needed
 ah_status nvrtc_compile_sm(int sm, const std::string& src, const char* name, std::vector<char>* cubin,
                            std::string* err);
-// Generated scan kernels, one process-wide cache keyed by source text: a kernel is compiled once,
+// Generated scan kernels, one process-wide cache keyed by patterns and shape: a kernel is compiled once,
 // callers that ask for it while it compiles wait for that compile.  Kernels stay loaded for the
 // life of the process.
 class JitCache {

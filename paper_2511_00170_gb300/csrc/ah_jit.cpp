@@ -1216,6 +1216,28 @@ ah_status load(int device, const std::vector<char>& cubin, int ops, const ScanCo
 
 }  // namespace
 
+namespace {
+
+// The architecture and everything a kernel's source is generated from: generating the source of a
+// one-pair kernel takes 1 ms, of an eight-pair one 8 ms, which a scan whose kernel is compiled already
+// need not spend again (a step on one contig took 0.72 ms with it).
+std::string kernel_key(int device, const std::vector<Pattern>& pats, const ScanConfig& cfg) {
+  int major = 0, minor = 0;
+  cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
+  cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
+  const int32_t f[] = {major * 10 + minor, cfg.threads,    cfg.groups_per_thread, cfg.shift_mode,  cfg.persistent,
+                       cfg.min_blocks,     cfg.emit_queue, cfg.vote_windows,      cfg.interleaved, cfg.il_rows};
+  std::string key((const char*)f, sizeof f);
+  for (const Pattern& P : pats) {
+    const uint8_t h[] = {P.len, P.clamp_lo, P.clamp_hi, P.k, (uint8_t)(P.id & 255), (uint8_t)(P.id >> 8)};
+    key.append((const char*)h, sizeof h);
+    key.append((const char*)P.set, P.len);
+  }
+  return key;
+}
+
+}  // namespace
+
 ah_status JitCache::get(ah_ctx* ctx, const std::vector<Pattern>& pats, const ScanConfig& cfg, ScanKernel* out) {
   std::string err;
   const ah_status st = get_impl(ctx->device, ctx, pats, cfg, out, &err, true);
@@ -1224,12 +1246,7 @@ ah_status JitCache::get(ah_ctx* ctx, const std::vector<Pattern>& pats, const Sca
 
 ah_status JitCache::get_impl(int device, ah_ctx* stats, const std::vector<Pattern>& pats, const ScanConfig& cfg,
                              ScanKernel* out, std::string* err_out, bool load_it) {
-  int ops = 0;
-  std::string src = scan_source(pats, cfg, &ops);
-  int major = 0, minor = 0;
-  cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
-  cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
-  const std::string key = std::to_string(major * 10 + minor) + "\n" + src;
+  const std::string key = kernel_key(device, pats, cfg);
   std::shared_ptr<Entry> e;
   bool mine = false;
   {
@@ -1247,7 +1264,8 @@ ah_status JitCache::get_impl(int device, ah_ctx* stats, const std::vector<Patter
     const auto t0 = std::chrono::steady_clock::now();
     std::vector<char> cubin;
     std::string err;
-    const ah_status st = compile(device, src, &cubin, &err);
+    int ops = 0;
+    const ah_status st = compile(device, scan_source(pats, cfg, &ops), &cubin, &err);
     {
       std::lock_guard<std::mutex> lock(e->m);
       e->st = st;
@@ -1376,12 +1394,8 @@ ah_status JitCache::prefetch(int device, ah_ctx* stats, const std::vector<std::v
 }
 
 bool JitCache::ready(int device, const std::vector<std::vector<Pattern>>& sets, const ScanConfig& cfg) {
-  int major = 0, minor = 0;
-  cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
-  cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
   for (const auto& pats : sets) {
-    int ops = 0;
-    const std::string key = std::to_string(major * 10 + minor) + "\n" + scan_source(pats, cfg, &ops);
+    const std::string key = kernel_key(device, pats, cfg);
     std::shared_ptr<Entry> e;
     {
       std::lock_guard<std::mutex> lock(mu_);

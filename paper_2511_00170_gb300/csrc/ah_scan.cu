@@ -272,6 +272,19 @@ __global__ void k_pair_offsets(const uint64_t* __restrict__ off, uint64_t n_tile
   if (p <= n_pairs) pair_off[p] = off[(uint64_t)p * n_tiles];
 }
 
+// What the host needs before it sizes a scan's output, written straight into page-locked memory: the
+// fullest tile, the status word, and (from word 2) every pair's first site, the last being the total.
+__global__ void k_scan_summary(const uint64_t* __restrict__ off, uint64_t n_tiles, uint32_t n_pairs,
+                               const uint32_t* __restrict__ tile_max, const uint32_t* __restrict__ status,
+                               uint64_t* __restrict__ pair_off, uint64_t* __restrict__ out) {
+  for (uint32_t p = threadIdx.x; p <= n_pairs; p += blockDim.x) {
+    const uint64_t v = off[(uint64_t)p * n_tiles];
+    pair_off[p] = v;
+    out[2 + p] = v;
+  }
+  if (threadIdx.x == 0) out[0] = *tile_max, out[1] = *status;
+}
+
 // ------------------------------------------------------------------------------------------
 // Generic scan: the same bit-sliced test with the primer set read from a table (GenPattern) at run
 // time, so a new primer set needs no compile.  Each position's mismatch bit is the two-variable
@@ -687,38 +700,60 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
   *out = nullptr;
   ScanConfig cfg = ctx->scan_cfg;
   const uint32_t n_pairs = p->n_pairs;
-  ah_status st;
-  uint64_t* slots = nullptr;
-  uint32_t* tile_count = nullptr;
-  uint32_t* d_max = nullptr;
-  if ((st = dalloc(ctx, &d_max, 1))) return st;
+  ah_status st = AH_OK;
+  uint64_t *slots = nullptr, *off = nullptr;
+  uint32_t *tile_count = nullptr, *d_max = nullptr, *tpc = nullptr, *big = nullptr;
+  ah_hits* h = new ah_hits();
+  h->ctx = ctx;
+  h->n_pairs = n_pairs;
+  auto release = [&] {
+    for (void* q : {(void*)slots, (void*)tile_count, (void*)tpc, (void*)off, (void*)big}) dfree(ctx, q);
+    slots = off = nullptr;
+    tile_count = tpc = big = nullptr;
+  };
+  auto done = [&](ah_status e) {
+    release();
+    dfree(ctx, d_max);
+    if (e) ah_hits_free(h);
+    else *out = h;
+    return e;
+  };
+  if ((st = dalloc(ctx, &d_max, 1)) || (st = dalloc(ctx, &h->d_pair_off, n_pairs + 1))) return done(st);
   uint64_t n_tiles = 0, tile_groups = 0;
   uint32_t cap = (uint32_t)cfg.slot_cap;
+  // The scan, the per-tile sort and the output positions in one go (the sort stops at a list's
+  // capacity, so an overflowed list is only wasted work), then one round trip for the sizes.
   for (;;) {
     tile_groups = scan_tile_groups(cfg);
     n_tiles = std::max<uint64_t>(1, (b->n_groups + tile_groups - 1) / tile_groups);
-    if ((st = dalloc(ctx, &slots, n_tiles * cap))) break;
-    if ((st = dalloc(ctx, &tile_count, n_tiles))) break;
-    AH_CUDA(ctx, cudaMemsetAsync(tile_count, 0, n_tiles * sizeof(uint32_t), ctx->stream));
-    AH_CUDA(ctx, cudaMemsetAsync(d_max, 0, sizeof(uint32_t), ctx->stream));
-    if ((st = launch_scan(ctx, b, p, cfg, per_record, tile_groups, n_tiles, slots, tile_count, cap))) break;
+    const uint64_t n_cells = (uint64_t)n_pairs * n_tiles;
+    if ((st = dalloc(ctx, &slots, n_tiles * cap)) || (st = dalloc(ctx, &tile_count, n_tiles)) ||
+        (st = dalloc(ctx, &tpc, n_cells)) || (st = dalloc(ctx, &off, n_cells + 1)) ||
+        (cap > kSmallTile && (st = dalloc(ctx, &big, n_tiles + 1))))
+      return done(st);
+    cudaMemsetAsync(tile_count, 0, n_tiles * sizeof(uint32_t), ctx->stream);
+    cudaMemsetAsync(d_max, 0, sizeof(uint32_t), ctx->stream);
+    cudaMemsetAsync(tpc, 0, n_cells * sizeof(uint32_t), ctx->stream);
+    if ((st = launch_scan(ctx, b, p, cfg, per_record, tile_groups, n_tiles, slots, tile_count, cap))) return done(st);
     launch_tile_max(ctx->stream, tile_count, n_tiles, d_max);
+    launched(ctx, 1 + launch_tile_sort(ctx->stream, slots, tile_count, cap, n_tiles, n_pairs, tpc, big, ctx->sm_count));
+    if ((st = exclusive_scan_u32(ctx, tpc, off, n_cells))) return done(st);
+    k_scan_summary<<<1, 256, 0, ctx->stream>>>(off, n_tiles, n_pairs, d_max, ctx->d_status, h->d_pair_off, ctx->h_read);
     launched(ctx);
-    AH_CUDA(ctx, cudaMemcpyAsync(ctx->h_status, d_max, 4, cudaMemcpyDeviceToHost, ctx->stream));
-    AH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    const uint32_t mx = *ctx->h_status;
-    *ctx->h_status = 0;
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) return done(fail(ctx, AH_ECUDA, "scan failed: %s", cudaGetErrorString(e)));
     if (ctx->timing) {
       float ms = 0.f;
-      AH_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]));
+      if (cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]) != cudaSuccess)
+        return done(fail(ctx, AH_ECUDA, "scan timing failed"));
       ctx->scan_ms += ms;
     }
+    if (ctx->h_read[1] && (st = check_status(ctx))) return done(st);
+    const uint32_t mx = (uint32_t)ctx->h_read[0];
     if (mx <= cap) break;
     // a tile overflowed: retry with room for the fullest tile, shrinking tiles when that is large
-    dfree(ctx, slots);
-    dfree(ctx, tile_count);
-    slots = nullptr;
-    tile_count = nullptr;
+    release();
     uint32_t need = 1;
     while (need < mx) need <<= 1;
     if (need <= 4096) {
@@ -728,57 +763,20 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
       if (cfg.interleaved) cfg.interleaved = 0;  // its tiles do not shrink
       if (cfg.groups_per_thread > 1) cfg.groups_per_thread = 1;
       else if (cfg.threads > 64) cfg.threads /= 2;
-      else return fail(ctx, AH_EOVERFLOW, "scan: more than %u sites in a tile of %d groups", mx, cfg.threads);
+      else return done(fail(ctx, AH_EOVERFLOW, "scan: more than %u sites in a tile of %d groups", mx, cfg.threads));
     }
   }
-  if (st) {
-    dfree(ctx, slots);
-    dfree(ctx, tile_count);
-    dfree(ctx, d_max);
-    return st;
+  h->h_pair_off.assign(ctx->h_read + 2, ctx->h_read + 3 + n_pairs);
+  h->n = h->h_pair_off[n_pairs];
+  if ((st = dalloc(ctx, &h->d, h->n))) return done(st);
+  if (h->n) {
+    k_emit_hits<<<(unsigned)((n_tiles + 7) / 8), 256, 0, ctx->stream>>>(slots, tile_count, cap, n_tiles, tile_groups, off,
+                                                                        b->rec_group, b->n_records, h->d);
+    launched(ctx);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return done(fail(ctx, AH_ECUDA, "site emission failed: %s", cudaGetErrorString(e)));
   }
-  // sort each tile, count per (pair, tile)
-  uint32_t* tpc = nullptr;
-  uint64_t* off = nullptr;
-  const uint64_t n_cells = (uint64_t)n_pairs * n_tiles;
-  if ((st = dalloc(ctx, &tpc, n_cells))) return st;
-  if ((st = dalloc(ctx, &off, n_cells + 1))) return st;
-  AH_CUDA(ctx, cudaMemsetAsync(tpc, 0, n_cells * sizeof(uint32_t), ctx->stream));
-  uint32_t* big = nullptr;  // tiles with more than 256 keys, sorted by the large-buffer kernel
-  if (cap > 256 && (st = dalloc(ctx, &big, n_tiles + 1))) return st;
-  const int sorts = launch_tile_sort(ctx->stream, slots, tile_count, cap, n_tiles, n_pairs, tpc, big, ctx->sm_count);
-  for (int i = 0; i < sorts; ++i) launched(ctx);
-  AH_CUDA(ctx, cudaGetLastError());
-  dfree(ctx, big);
-  if ((st = exclusive_scan_u32(ctx, tpc, off, n_cells))) return st;
-  uint64_t total = 0;
-  if ((st = read_u64(ctx, off + n_cells, &total))) return st;
-  ah_hits* h = new ah_hits();
-  h->ctx = ctx;
-  h->n = total;
-  h->n_pairs = n_pairs;
-  if ((st = dalloc(ctx, &h->d, total)) || (st = dalloc(ctx, &h->d_pair_off, n_pairs + 1))) {
-    ah_hits_free(h);
-    return st;
-  }
-  launch_emit_hits(ctx->stream, slots, tile_count, cap, n_tiles, tile_groups, off, b, h->d, nullptr, ~0ull, nullptr,
-                   h->d_pair_off, n_pairs);
-  launched(ctx, 2);
-  AH_CUDA(ctx, cudaGetLastError());
-  h->h_pair_off.resize(n_pairs + 1);
-  AH_CUDA(ctx, cudaMemcpyAsync(h->h_pair_off.data(), h->d_pair_off, (n_pairs + 1) * sizeof(uint64_t),
-                               cudaMemcpyDeviceToHost, ctx->stream));
-  dfree(ctx, slots);
-  dfree(ctx, tile_count);
-  dfree(ctx, d_max);
-  dfree(ctx, tpc);
-  dfree(ctx, off);
-  if ((st = check_status(ctx))) {
-    ah_hits_free(h);
-    return st;
-  }
-  *out = h;
-  return AH_OK;
+  return done(AH_OK);
 }
 
 }  // namespace

@@ -2015,9 +2015,12 @@ ah_status tm_filter(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const a
     uint64_t* off;
     if ((st = dalloc(ctx, &off, a->n + 1))) return st;
     if ((st = exclusive_scan_u32(ctx, keep, off, a->n))) return st;
+    // the number kept and the status word in one round trip
+    AH_CUDA(ctx, cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
     uint64_t kept = 0;
     if ((st = read_u64(ctx, off + a->n, &kept))) return st;
-    ah_amplicon* nd;
+    const bool flagged = *ctx->h_status != 0;
+    ah_amplicon* nd = nullptr;
     if ((st = dalloc(ctx, &nd, kept))) return st;
     if (a->n)
       k_compact_amps<<<(unsigned)((a->n + 255) / 256), 256, 0, ctx->stream>>>(a->d, a->n, keep, off, nd);
@@ -2027,9 +2030,12 @@ ah_status tm_filter(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const a
     dfree(ctx, off);
     a->d = nd;
     a->n = kept;
+    dfree(ctx, hit_tm);
+    dfree(ctx, keep);
+    dfree(ctx, defer);
+    return flagged ? check_status(ctx) : AH_OK;
   }
   dfree(ctx, hit_tm);
-  dfree(ctx, keep);
   dfree(ctx, defer);
   return check_status(ctx);
 }

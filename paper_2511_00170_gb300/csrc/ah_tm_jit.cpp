@@ -398,15 +398,21 @@ std::vector<std::string> primer_list(const ah_primers* p) {
   return v;
 }
 
-// compiles (once per source) and, when load_it, loads the kernel; err filled on failure
-ah_status get_kernel(int device, ah_ctx* stats, const std::vector<std::string>& primers, bool load_it, TmKernel* out,
-                     std::string* err) {
-  int words = 0;
-  const std::string src = tm_chain_source(primers, &words);
+// The architecture and the primers, which the source is generated from (generating it again for a
+// kernel that is compiled already would take longer than a small step's Tm).
+std::string kernel_key(int device, const std::vector<std::string>& primers) {
   int major = 0, minor = 0;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
-  const std::string key = std::to_string(major * 10 + minor) + "\n" + src;
+  std::string key = std::to_string(major * 10 + minor);
+  for (const std::string& p : primers) key += "\n" + p;
+  return key;
+}
+
+// compiles (once per primer list) and, when load_it, loads the kernel; err filled on failure
+ah_status get_kernel(int device, ah_ctx* stats, const std::vector<std::string>& primers, bool load_it, TmKernel* out,
+                     std::string* err) {
+  const std::string key = kernel_key(device, primers);
   std::shared_ptr<TmEntry> e;
   bool mine = false;
   {
@@ -424,6 +430,8 @@ ah_status get_kernel(int device, ah_ctx* stats, const std::vector<std::string>& 
     const auto t0 = std::chrono::steady_clock::now();
     std::vector<char> cubin;
     std::string cerr;
+    int words = 0;
+    const std::string src = tm_chain_source(primers, &words);
     const ah_status st = nvrtc_compile(device, src, "ah_tm_jit.cu", &cubin, &cerr);
     {
       std::lock_guard<std::mutex> lock(e->m);
@@ -470,11 +478,7 @@ enum Lookup { kAbsent, kBusy, kReady };
 
 // the kernel if it is compiled (loading it into the process here when it was compiled elsewhere)
 Lookup lookup(int device, const std::vector<std::string>& primers, TmKernel* out) {
-  const std::string src = tm_chain_source(primers, nullptr);
-  int major = 0, minor = 0;
-  cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
-  cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
-  const std::string key = std::to_string(major * 10 + minor) + "\n" + src;
+  const std::string key = kernel_key(device, primers);
   std::shared_ptr<TmEntry> e;
   {
     std::lock_guard<std::mutex> lock(g_mu);
