@@ -824,6 +824,66 @@ __device__ bool group_viterbi(const TmGroupSh& sh, const int32_t* __restrict__ w
   return true;
 }
 
+// The n-th set bit of a choice set.
+__device__ __forceinline__ int nth_choice(uint32_t ch, uint32_t n) {
+  for (uint32_t i = 0; i < n; ++i) ch &= ch - 1;
+  return __ffs(ch) - 1;
+}
+
+// Maximum Tm over the qualifying variants of a compressed chain, enumerated by the group's lanes: lane
+// r takes combinations r, r + G, ... of the choices at the branch positions (the digits of the
+// combination's number), sums their weights, and evaluates the Tm of those within the mismatch budget
+// (m0: the fixed positions' mismatches, gc0: their G/C count).  For the salt methods whose
+// correction depends on each variant's G/C content, where no chain iteration applies.  Sums are exact
+// and a variant's Tm is the walk's (enum_max), so the maximum is the same number.
+//
+// FP64 runs at a sixteenth of a warp instruction per cycle, so a variant is evaluated in single
+// precision first and skipped when that lies 0.05 K below the best so far: with |dS| above 50 and
+// temperatures below 2,000 K rounding moves it by 3e-6 of itself, 0.006 K, at most.
+// With one lane walking a site's variants position by position, ah_tm_filter took 2,202 us for the
+// 6,200 sites of four pairs (up to 128 combinations each) on 60 Mbp of contigs; with this 296 us.
+constexpr uint32_t kTmGroupEnum = 2048;  // combinations; sites with more keep the walk, which prunes
+template <int G>
+__device__ double group_enum_max(const TmGroupSh& sh, const int32_t* __restrict__ w, int D, uint32_t combos, int K,
+                                 int m0, int gc0, int L, const TmRun& R, int r, unsigned gmask) {
+  const float h0 = (float)R.init_h, s0 = (float)(R.init_s + R.sym_s + R.rlnk), h1 = (float)R.sym_h;
+  double best = -INFINITY;
+  bool any = false;
+  for (uint32_t x = (uint32_t)r; x < combos; x += G) {
+    uint32_t rest = x;
+    int32_t sum = 0;
+    int mm = m0, gc = gc0, a = 0;
+    for (int t = 0; t < D; ++t) {
+      const int j = sh.dpos[t];
+      const uint32_t ch = sh.ch[j];
+      const uint32_t n = (uint32_t)__popc(ch);
+      const uint32_t q = n == 3 ? rest * 0xAAABu >> 17 : rest >> (n >> 1);  // rest / n for n = 1..4
+      const int b = nth_choice(ch, rest - q * n);
+      rest = q;
+      sum = t == 0 ? sh.pre[b] : add_packed(sum, w[(t - 1) * 16 + a * 4 + b]);
+      mm += K >= 0 && b != sh.s[j];
+      gc += b & 1;
+      a = b;
+    }
+    sum = add_packed(sum, sh.suf[a]);
+    if (sum == kNoEdge || (K >= 0 && mm > K)) continue;
+    const int dh10 = unpack_dh(sum), ds10 = unpack_ds(sum);
+    any = true;
+    const float dh = 0.1f * (float)dh10 + h0 + h1 + (float)(gc ? R.onegc_h : R.allat_h);
+    const float ds = 0.1f * (float)ds10 + s0 + (float)(gc ? R.onegc_s : R.allat_s);
+    const float tk = 1000.f * dh / ds;
+    if (ds < -50.f && fabsf(tk) < 2000.f) {
+      const float corr = (float)R.rc0 + (float)R.rc1 * ((float)gc / (float)L) + (float)R.rc2 / (2.f * (float)(L - 1));
+      const float inv = 1.f / tk + corr;
+      if (fabsf(inv) > 5e-4f && 1.f / inv - 273.15f < (float)best - 0.05f) continue;
+    }
+    best = fmax(best, tm_of_tenths(dh10, ds10, gc, L, R));
+  }
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(gmask, best, o, G));
+  return __any_sync(gmask, any) ? best : __longlong_as_double(0x7ff8000000000000ll);
+}
+
 // Tm of the site held in sh (set, s and c filled, L its length) for a primer with mismatch budget k
 // (k >= L: none) and clamp: the maximum over qualifying variants, as site_tm returns it.  Called by
 // all G lanes of the group (lane r, mask gmask); w: the group's weight area (room for dmax - 1 steps).
@@ -833,7 +893,7 @@ __device__ double group_site_tm(TmGroupSh& sh, int32_t* w, int L, int k, int cla
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
   const int K = k >= L ? -1 : k, W = K < 0 ? 1 : K + 1;
   // choices per position, the branch positions, and the fixed positions' mismatches
-  uint32_t dmask = 0, empty = 0, fixed_mm = 0;
+  uint32_t dmask = 0, empty = 0, fixed_mm = 0, fixed_gc = 0;
   for (int j = r; j < L; j += G) {
     uint8_t ch = sh.set[j];
     if (j >= L - clamp) ch &= (uint8_t)(1u << sh.s[j]);
@@ -842,17 +902,24 @@ __device__ double group_site_tm(TmGroupSh& sh, int32_t* w, int L, int k, int cla
     if (n == 0) empty |= 1u << j;
     if (n >= 2) dmask |= 1u << j;
     if (n == 1 && K >= 0 && ch != (1u << sh.s[j])) fixed_mm |= 1u << j;
+    if (n == 1 && (fixed_base(ch) & 1)) fixed_gc |= 1u << j;
   }
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) {
     dmask |= __shfl_xor_sync(gmask, dmask, o, G);
     empty |= __shfl_xor_sync(gmask, empty, o, G);
     fixed_mm |= __shfl_xor_sync(gmask, fixed_mm, o, G);
+    fixed_gc |= __shfl_xor_sync(gmask, fixed_gc, o, G);
   }
   if (empty) return nan;
   const int m0 = __popc(fixed_mm);
   if (K >= 0 && m0 > K) return nan;
-  if (R.saltcorr >= 6 || L < 3 || W * 4 > G || R.gc_split) {
+  __syncwarp(gmask);  // ch is read by the whole group
+  const bool flat = R.saltcorr >= 6 && L >= 3;  // enumerated by the group, unless too many combinations
+  uint32_t combos = 1;
+  if (flat)
+    for (uint32_t x = dmask; x && combos <= kTmGroupEnum; x &= x - 1) combos *= __popc(sh.ch[__ffs(x) - 1]);
+  if (L < 3 || (flat ? combos > kTmGroupEnum : W * 4 > G || R.gc_split)) {
     __syncwarp(gmask);
     double t = nan;
     if (r == 0) t = site_tm(sh.set, sh.s, L, k, clamp, R, status);
@@ -923,6 +990,7 @@ __device__ double group_site_tm(TmGroupSh& sh, int32_t* w, int L, int k, int cla
     }
   }
   __syncwarp(gmask);
+  if (flat) return group_enum_max<G>(sh, w, D, combos, K, __popc(fixed_mm & ~dmask), __popc(fixed_gc & ~dmask), L, R, r, gmask);
   // a bound on every variant's dS: each step's largest (tenths)
   int bound = 0;
   for (int t = r; t + 1 < D; t += G) {
@@ -1066,8 +1134,8 @@ __device__ __forceinline__ bool edge_defined(const NNTablesI& ti, int i, int L, 
   return __ldg(&ti.step_h[x * 64 + y * 16 + c0 * 4 + c1]) != kNoParam;
 }
 
-// The group-per-site form of k_tm_hits.  A block takes a window of kTmWindow site slots, one per
-// thread.  Each thread first settles its slot where that needs no chain: not wanted (no amplicon
+// The group-per-site form of k_tm_hits.  A block takes a window of `window` site slots (at most
+// kTmWindow), one per thread.  Each thread first settles its slot where that needs no chain: not wanted (no amplicon
 // pairs it), or undefined (a site base outside the clamp's choice, too many fixed mismatches, or a
 // step between single-choice positions without a parameter; the group repeats these checks).  The
 // remaining sites are sorted by primer (so neighbouring groups walk chains of one shape) and taken
@@ -1083,7 +1151,7 @@ __global__ void __launch_bounds__(kTmWindow) k_tm_hits_g(const ah_hit* __restric
                                                          const uint8_t* __restrict__ psets,
                                                          const uint8_t* __restrict__ pk, int clamp, const TmRun Rp,
                                                          double* __restrict__ out, uint32_t* status, int dmax,
-                                                         int n_groups, const uint64_t* __restrict__ d_n) {
+                                                         int n_groups, int window, const uint64_t* __restrict__ d_n) {
   // the run constants in shared memory: device functions take them by reference, and a reference
   // to a kernel parameter would make the compiler copy it to local memory for every thread
   __shared__ TmRun R_sh;
@@ -1096,13 +1164,13 @@ __global__ void __launch_bounds__(kTmWindow) k_tm_hits_g(const ah_hit* __restric
   uint64_t* codes = reinterpret_cast<uint64_t*>(tm_smem + kTmWindow);  // kTmWindow
   uint32_t* areas = tm_smem + 3 * kTmWindow;
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
-  const uint64_t base = (uint64_t)blockIdx.x * kTmWindow;
+  const uint64_t base = (uint64_t)blockIdx.x * (uint32_t)window;
   const uint64_t n_here = d_n ? min(n, *d_n) : n;
   {
     const int t = threadIdx.x;
     const uint64_t i = base + t;
     uint32_t key = 0xFFFFFFFFu;
-    if (i < n_here && (unsigned long long)__double_as_longlong(out[i]) == kSiteWanted) {
+    if (t < window && i < n_here && (unsigned long long)__double_as_longlong(out[i]) == kSiteWanted) {
       const ah_hit h = hits[i];
       const int L = plen[h.pattern];
       const uint32_t pair = h.pattern >> 2, primer = h.pattern & 1u, strand = (h.pattern >> 1) & 1u;
@@ -1836,10 +1904,15 @@ int launch_tm_hits(cudaStream_t s, const TmRun& R, const ah_primers* p, const ah
         hits, cap, planes, rec_group, p->d_plen, p->d_psets, p->d_pk, p->clamp, R, hit_tm, status, d_n);
     return 1;
   }
-  const unsigned grid = (unsigned)std::max<uint64_t>(1, (cap + kTmWindow - 1) / kTmWindow);
+  // few sites: smaller windows, down to two rounds of the block's groups, until four blocks per SM have
+  // work (a block takes its sites in rounds, one after another; ah_tm_filter on the 6,200 sites of
+  // four pairs on 60 Mbp of contigs: 296 us with windows of 128, 84 us with the smaller ones)
+  int window = kTmWindow;
+  while (window > 2 * t.S && cap < 4ull * (uint64_t)std::max(1, sm_count) * (uint64_t)window) window /= 2;
+  const unsigned grid = (unsigned)std::max<uint64_t>(1, (cap + window - 1) / window);
 #define AH_TM_HITS_G(GG)                                                                                        \
   k_tm_hits_g<GG><<<grid, kTmWindow, t.smem, s>>>(hits, cap, planes, rec_group, p->d_plen, p->d_psets, p->d_pk, \
-                                                  p->clamp, R, hit_tm, status, t.dmax, t.S, d_n)
+                                                  p->clamp, R, hit_tm, status, t.dmax, t.S, window, d_n)
   switch (t.G) {
     case 4: AH_TM_HITS_G(4); break;
     case 8: AH_TM_HITS_G(8); break;
