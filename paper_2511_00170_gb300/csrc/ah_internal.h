@@ -118,6 +118,7 @@ struct ah_ctx {
   cudaMemPool_t pool = nullptr;      // the context's stream-ordered memory pool
   uint8_t* bounce[2] = {nullptr, nullptr};       // page-locked buffers for copies into pageable memory
   cudaEvent_t bounce_ev[2] = {nullptr, nullptr};
+  bool stage_pending = false;        // an upload from bounce[0] may be in flight (its end: bounce_ev[0])
   uint32_t* d_status = nullptr;      // device status word
   uint32_t* h_status = nullptr;      // pinned mirror
   uint64_t* h_read = nullptr;        // page-locked words for counts read back (kReadWords)
@@ -253,6 +254,8 @@ ah_status exclusive_scan_u64(ah_ctx* ctx, const uint64_t* d_in, uint64_t* d_out,
 // pageable path (one staging pipeline for every stream of the process)
 ah_status copy_to_host(ah_ctx* ctx, void* dst, const void* src, uint64_t bytes);
 constexpr uint64_t kBounceBytes = 8ull << 20;  // each of a context's two bounce buffers
+// both bounce buffers allocated, and no upload from the first in flight
+ah_status stage_buffer(ah_ctx* ctx);
 constexpr int kReadWords = 512;  // page-locked words of a context for counts read back
 // read one uint64 (or n of them, at most 8, from places of their own) from device memory through the
 // context's page-locked words, in one synchronisation of the stream

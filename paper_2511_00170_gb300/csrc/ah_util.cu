@@ -23,6 +23,16 @@ void dfree(ah_ctx* ctx, void* p) {
   if (p) cudaFreeAsync(p, ctx->stream);
 }
 
+ah_status stage_buffer(ah_ctx* ctx) {
+  for (int b = 0; b < 2; ++b) {
+    if (!ctx->bounce[b]) AH_CUDA(ctx, cudaMallocHost(&ctx->bounce[b], kBounceBytes));
+    if (!ctx->bounce_ev[b]) AH_CUDA(ctx, cudaEventCreateWithFlags(&ctx->bounce_ev[b], cudaEventDisableTiming));
+  }
+  if (ctx->stage_pending) AH_CUDA(ctx, cudaEventSynchronize(ctx->bounce_ev[0]));
+  ctx->stage_pending = false;
+  return AH_OK;
+}
+
 ah_status copy_to_host(ah_ctx* ctx, void* dst, const void* src, uint64_t bytes) {
   if (bytes) {
     cudaPointerAttributes pa;
@@ -31,10 +41,8 @@ ah_status copy_to_host(ah_ctx* ctx, void* dst, const void* src, uint64_t bytes) 
     if (locked || bytes <= (64u << 10)) {
       AH_CUDA(ctx, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, ctx->stream));
     } else {
-      for (int b = 0; b < 2; ++b) {
-        if (!ctx->bounce[b]) AH_CUDA(ctx, cudaMallocHost(&ctx->bounce[b], kBounceBytes));
-        if (!ctx->bounce_ev[b]) AH_CUDA(ctx, cudaEventCreateWithFlags(&ctx->bounce_ev[b], cudaEventDisableTiming));
-      }
+      const ah_status st = stage_buffer(ctx);
+      if (st) return st;
       // chunk i lands in buffer i % 2 while the host copies chunk i - 1 out of the other
       uint64_t off[2] = {0, 0}, len[2] = {0, 0};
       int i = 0;
