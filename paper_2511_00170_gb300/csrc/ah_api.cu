@@ -844,7 +844,9 @@ ah_status ah_pack_batch_device(ah_ctx* ctx, uint32_t n_rec, const uint8_t* d_seq
   ah_status st = layout_batch(ctx, n_rec, lens.data(), genome_ids, b, h_offsets, &d_rank);
   if (!st) {
     launch_pack_records(ctx, d_seq, d_rank, b);
-    if (cudaGetLastError() != cudaSuccess) st = fail(ctx, AH_ECUDA, "ah_pack_batch_device: launch failed");
+    // another context's stream may read the batch, and the caller may free d_seq, once this returns
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+      st = fail(ctx, AH_ECUDA, "ah_pack_batch_device: packing failed");
   }
   dfree(ctx, d_rank);
   if (st) {
