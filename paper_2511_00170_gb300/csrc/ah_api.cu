@@ -363,6 +363,32 @@ uint8_t set_complement(uint8_t s) {
 // ------------------------------------------------------------------------------------------
 namespace ah {
 
+ah_status pack_device_records(ah_ctx* ctx, uint32_t n_rec, const uint8_t* d_seq, const uint64_t* h_offsets,
+                              const uint32_t* genome_ids, ah_batch** out) {
+  *out = nullptr;
+  cudaSetDevice(ctx->device);
+  std::vector<uint64_t> lens(n_rec);
+  for (uint32_t r = 0; r < n_rec; ++r) {
+    if (h_offsets[r + 1] < h_offsets[r]) return fail(ctx, AH_EINVAL, "ah_pack_batch_device: offsets decrease");
+    lens[r] = h_offsets[r + 1] - h_offsets[r];
+  }
+  ah_batch* b = new ah_batch();
+  uint64_t* d_rank = nullptr;
+  ah_status st = layout_batch(ctx, n_rec, lens.data(), genome_ids, b, h_offsets, &d_rank);
+  if (!st) {
+    launch_pack_records(ctx, d_seq, d_rank, b);
+    if (cudaGetLastError() != cudaSuccess) st = fail(ctx, AH_ECUDA, "ah_pack_batch_device: launch failed");
+  }
+  dfree(ctx, d_rank);
+  if (st) {
+    free_batch_arrays(b);
+    delete b;
+    return st;
+  }
+  *out = b;
+  return AH_OK;
+}
+
 ah_status pack_batch_ranked(ah_ctx* ctx, uint32_t n, const uint8_t* d_seq, const uint64_t* d_rank,
                             const uint64_t* h_rank, const uint32_t* genome_ids, ah_batch** out) {
   *out = nullptr;
@@ -832,29 +858,14 @@ ah_status ah_pack_batch(ah_ctx* ctx, uint32_t n_rec, const char* const* seqs, co
 ah_status ah_pack_batch_device(ah_ctx* ctx, uint32_t n_rec, const uint8_t* d_seq, const uint64_t* h_offsets,
                                const uint32_t* genome_ids, ah_batch** out) {
   if (!ctx || !out || !h_offsets || n_rec == 0 || !d_seq) return fail(ctx, AH_EINVAL, "ah_pack_batch_device: bad arguments");
-  *out = nullptr;
-  cudaSetDevice(ctx->device);
-  std::vector<uint64_t> lens(n_rec);
-  for (uint32_t r = 0; r < n_rec; ++r) {
-    if (h_offsets[r + 1] < h_offsets[r]) return fail(ctx, AH_EINVAL, "ah_pack_batch_device: offsets decrease");
-    lens[r] = h_offsets[r + 1] - h_offsets[r];
+  const ah_status st = pack_device_records(ctx, n_rec, d_seq, h_offsets, genome_ids, out);
+  if (st) return st;
+  // another context's stream may read the batch, and the caller may free d_seq, once this returns
+  if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
+    ah_batch_free(*out);
+    *out = nullptr;
+    return fail(ctx, AH_ECUDA, "ah_pack_batch_device: packing failed");
   }
-  ah_batch* b = new ah_batch();
-  uint64_t* d_rank = nullptr;
-  ah_status st = layout_batch(ctx, n_rec, lens.data(), genome_ids, b, h_offsets, &d_rank);
-  if (!st) {
-    launch_pack_records(ctx, d_seq, d_rank, b);
-    // another context's stream may read the batch, and the caller may free d_seq, once this returns
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(ctx->stream) != cudaSuccess)
-      st = fail(ctx, AH_ECUDA, "ah_pack_batch_device: packing failed");
-  }
-  dfree(ctx, d_rank);
-  if (st) {
-    free_batch_arrays(b);
-    delete b;
-    return st;
-  }
-  *out = b;
   return AH_OK;
 }
 

@@ -261,10 +261,14 @@ constexpr int kReadWords = 512;  // page-locked words of a context for counts re
 // context's page-locked words, in one synchronisation of the stream
 ah_status read_u64(ah_ctx* ctx, const uint64_t* d, uint64_t* h);
 ah_status read_u64s(ah_ctx* ctx, int n, const uint64_t* const* d, uint64_t* const* h);
+// ah_pack_batch_device without its wait: d_seq must stay until ctx->stream has passed the packing.
+ah_status pack_device_records(ah_ctx* ctx, uint32_t n_rec, const uint8_t* d_seq, const uint64_t* h_offsets,
+                              const uint32_t* genome_ids, ah_batch** out);
 // A batch of n records whose bases lie in device memory at d_seq[rank[r], rank[r + 1]) (rank[n] =
 // total), with the ranks both on the device (d_rank, n values) and on the host (h_rank, n + 1
-// values).  Lengths, group offsets and packing items are computed on the device; the batch's host
-// record table from h_rank; no per-record array crosses the host link.  The caller has checked that
+// values; its first n may still be on their way by a copy on ctx->stream, the last is there).
+// Lengths and group offsets are computed on the device; the batch's host record table from h_rank; no
+// per-record array crosses the host link.  The caller has checked that
 // the ranks do not decrease and that every record is shorter than 2^32 bases (the device reads each
 // record's bytes by them).  Synchronises.
 ah_status pack_batch_ranked(ah_ctx* ctx, uint32_t n, const uint8_t* d_seq, const uint64_t* d_rank,
