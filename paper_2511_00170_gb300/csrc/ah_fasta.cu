@@ -592,17 +592,10 @@ __global__ void k_rank_offsets(const uint64_t* __restrict__ rank, uint64_t n, ui
   if (r <= n) off[r] = (r < n ? rank[r] : total) - rank[0];
 }
 
-// The tiles of the next chunk when rest are left.  Host text is copied and parsed in chunks of half of what is
-// left, so that a chunk's passes run while the next crosses the link and little is parsed after the last byte has
-// landed: at least `least` bytes (a chunk costs some 25 us of launches, waits and chaining), at most kChunkBases.
-// 98 MB took 614 us in four equal chunks, 699 in eight, 980 in sixteen, 530 in four halving ones (the copy alone
-// 487).
+// Tiles of the next chunk of host text when rest are left: half of it (98 MB of FASTA took 614 us in four equal chunks,
+// 699 in eight, 980 in sixteen, 530 this way; three quarters and 8 MiB at least 30 more; the copy alone 487).
 constexpr uint64_t kLeastChunk = 12ull << 20, kLeastHookChunk = 32ull << 20;  // (a hook waits for each chunk)
-uint64_t next_chunk(uint64_t rest, uint64_t least) {
-  const uint64_t least_tiles = least / kFaTile;
-  if (rest <= least_tiles + least_tiles / 2) return rest;
-  return std::min<uint64_t>(kChunkBases / kFaTile, std::max<uint64_t>(least_tiles, rest / 2));
-}
+uint64_t next_tiles(uint64_t rest, uint64_t least) { return next_chunk(rest, least / kFaTile, kChunkBases / kFaTile, 4); }
 
 }  // namespace
 }  // namespace ah
@@ -703,7 +696,7 @@ ah_status fasta_pack(ah_ctx* ctx, const char* text, uint64_t n_bytes, const uint
     // all of them at once; from pageable memory a copy returns once it is staged, and the chunk's passes
     // are enqueued before the next.
     for (uint64_t t0 = 0, nt; t0 < n_tiles && !st; t0 += nt) {
-      nt = on_device ? n_tiles : next_chunk(n_tiles - t0, hook ? kLeastHookChunk : kLeastChunk);
+      nt = on_device ? n_tiles : next_tiles(n_tiles - t0, hook ? kLeastHookChunk : kLeastChunk);
       const uint64_t b0 = t0 * kFaTile, nb = std::min(n_bytes, b0 + nt * kFaTile) - b0;
       if (!on_device) {
         cudaEvent_t e = nullptr;
@@ -955,7 +948,7 @@ ah_status ah_fastq_pack(ah_ctx* ctx, const char* text, uint64_t n_bytes, const u
       t = staged;
     }
     for (uint64_t t0 = 0, nt; t0 < n_tiles && !st; t0 += nt) {
-      nt = on_device ? n_tiles : next_chunk(n_tiles - t0, kLeastChunk);
+      nt = on_device ? n_tiles : next_tiles(n_tiles - t0, kLeastChunk);
       if (!on_device) {
         const uint64_t b0 = t0 * kFaTile, nb = std::min(n_bytes, b0 + nt * kFaTile) - b0;
         cudaEvent_t e = nullptr;

@@ -253,6 +253,13 @@ ah_status exclusive_scan_u64(ah_ctx* ctx, const uint64_t* d_in, uint64_t* d_out,
 // ones through the context's two page-locked bounce buffers, so that no copy takes the driver's
 // pageable path (one staging pipeline for every stream of the process)
 ah_status copy_to_host(ah_ctx* ctx, void* dst, const void* src, uint64_t bytes);
+// Host data is copied and worked on in chunks.  How much of the `rest` left the next chunk takes: `eighths` of it, so
+// that a chunk's work is done by the time the rest has crossed the link and little is left to do after the last byte;
+// at least `least` (a chunk costs some 10 to 25 us of launches, waits and a shorter copy), at most `most`.
+inline uint64_t next_chunk(uint64_t rest, uint64_t least, uint64_t most, uint64_t eighths) {
+  if (rest <= least + least / 2) return rest;
+  return std::min(most, std::max(least, rest / 8 * eighths));
+}
 constexpr uint64_t kBounceBytes = 8ull << 20;  // each of a context's two bounce buffers
 // both bounce buffers allocated, and no upload from the first in flight
 ah_status stage_buffer(ah_ctx* ctx);

@@ -572,14 +572,12 @@ ah_status ah_plan_launch_packed(ah_plan* pl, const void* h_planes, uint64_t n_in
   // the invalid words first (a small list), then the planes in chunks of kChunkBases bases on a
   // copy stream straight into the batch; each range of scan tiles whose groups (and the group after
   // them) have landed is scanned while the next chunk crosses the link
-  const uint64_t chunk = kChunkBases / kGroupBases;  // groups per copy (64 MiB of planes)
-  const uint64_t n_chunks = (b->n_groups + chunk - 1) / chunk;
+  const uint64_t chunk = kChunkBases / kGroupBases;  // groups per copy at most (64 MiB of planes)
   cudaStream_t cs = nullptr;
   cudaEvent_t ready = nullptr;
-  std::vector<cudaEvent_t> landed(n_chunks, nullptr);
+  std::vector<cudaEvent_t> landed;
   cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
-  for (uint64_t k = 0; k < n_chunks && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&landed[k], cudaEventDisableTiming);
   // the sparse list crosses the link first (the planes' chunks would queue it behind them on the copy
   // engine); the plane copies wait for earlier work that may still read the planes, and the invalid
   // words are written by kernels meanwhile (only the scans read them)
@@ -590,12 +588,16 @@ ah_status ah_plan_launch_packed(ah_plan* pl, const void* h_planes, uint64_t n_in
   if (e == cudaSuccess && (st = scatter_invalid_list(c, b, &il))) e = cudaErrorUnknown;
   const uint64_t tg = pl->range_kern.tile_groups;
   uint64_t scanned = 0, scan_launches = 0;
-  for (uint64_t k = 0; k < n_chunks && e == cudaSuccess; ++k) {
-    const uint64_t g0 = k * chunk, g1 = std::min(b->n_groups, g0 + chunk);
-    e = cudaMemcpyAsync(b->planes + g0, (const uint2*)h_planes + g0, (g1 - g0) * sizeof(uint2), cudaMemcpyHostToDevice,
-                        cs);
-    if (e == cudaSuccess) e = cudaEventRecord(landed[k], cs);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, landed[k], 0);
+  for (uint64_t g0 = 0, g1; g0 < b->n_groups && e == cudaSuccess; g0 = g1) {
+    // (4 MiB at least; a chunk's scan takes a sixth of its copy's time)
+    g1 = g0 + next_chunk(b->n_groups - g0, 1ull << 19, chunk, 6);
+    landed.push_back(nullptr);
+    e = cudaEventCreateWithFlags(&landed.back(), cudaEventDisableTiming);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(b->planes + g0, (const uint2*)h_planes + g0, (g1 - g0) * sizeof(uint2), cudaMemcpyHostToDevice,
+                          cs);
+    if (e == cudaSuccess) e = cudaEventRecord(landed.back(), cs);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, landed.back(), 0);
     const uint64_t upto = g1 >= b->n_groups ? b->n_groups : (g1 - 1) / tg * tg;
     if (e == cudaSuccess && upto > scanned) {
       launch_scan_range(c->stream, pl->range_kern, b, pl->slots, pl->tile_count, pl->slot_cap, c->d_status, scanned,
