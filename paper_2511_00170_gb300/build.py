@@ -20,7 +20,7 @@ SOURCES = ["ah_api.cu", "ah_util.cu", "ah_scan.cu", "ah_pair.cu", "ah_tm.cu", "a
            "ah_tm_jit.cpp", "ah_serve.cpp", "ah_output.cpp", "ah_files.cpp"]
 # headers every translation unit may include; ah_tm_chain.cuh is also compiled at run time (its text
 # is embedded in the library by _embed)
-HEADERS = ["ah_internal.h", "ah_tm_chain.cuh"]
+HEADERS = ["ah_internal.h", "ah_amps.cuh", "ah_tm_chain.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -5,6 +5,7 @@
 // reverse barcode, site i and site j in primer orientation.  A length pass and an exclusive scan
 // place every amplicon; then blocks decode the fields of consecutive amplicons from the 2-bit planes,
 // an aligned 16-byte unit of the arena per thread.
+#include "ah_amps.cuh"
 #include "ah_internal.h"
 
 namespace ah {
@@ -198,6 +199,60 @@ __global__ void __launch_bounds__(kExThreads) k_extract_write(
 
 unsigned extract_blocks(uint64_t n) { return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(kExBlocks, (n + kExMinAmps - 1) / kExMinAmps)); }
 
+// What follows the Tm stage in one block for up to kOneBlockItems amplicons: threshold, compaction (with the filter) and,
+// with ebase, the bytes of each kept amplicon and their offsets.  4 kept of 26 amplicons took 36 us in nine kernels, 7.4
+// here.
+constexpr int kOneThreads = 1024;
+__global__ void __launch_bounds__(kOneThreads) k_finish_one(
+    ah_amplicon* __restrict__ amps, uint64_t cap, const uint64_t* __restrict__ d_n, const double* __restrict__ hit_tm,
+    int filter, double min_tm, ah_amplicon* __restrict__ kept, uint64_t* __restrict__ n_kept,
+    const ah_hit* __restrict__ hits, const uint32_t* __restrict__ rec_len, const uint8_t* __restrict__ plen, int trim,
+    int64_t fb, int64_t rb, uint64_t* __restrict__ ebase) {
+  __shared__ uint64_t bytes_of[kOneThreads / 32];
+  __shared__ uint32_t kept_of[kOneThreads / 32];
+  const uint64_t n = min(*d_n, cap);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint64_t n_out = 0, n_bytes = 0;
+  for (uint64_t base = 0; base < n; base += kOneThreads) {
+    const uint64_t i = base + threadIdx.x;
+    ah_amplicon m{};
+    bool keep = false;
+    uint64_t len = 0;
+    if (i < n) {
+      m = amps[i];
+      keep = decide_amplicon(&m, hit_tm[m.hit_i], hit_tm[m.hit_j], min_tm) || !filter;
+      amps[i] = m;
+      if (keep && ebase) {
+        const Fields f = fields_of(m, hits[m.hit_i], hits[m.hit_j], plen, rec_len[m.record], trim, fb, rb);
+        for (int q = 0; q < 5; ++q) len += (uint64_t)(f.b[q] - f.a[q]);
+      }
+    }
+    const uint32_t votes = __ballot_sync(0xffffffffu, keep);
+    uint64_t inc = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) bytes_of[warp] = inc, kept_of[warp] = __popc(votes);
+    __syncthreads();
+    uint64_t at = n_bytes + inc - len, k = n_out + __popc(votes & ((1u << lane) - 1u));
+    for (int w = 0; w < kOneThreads / 32; ++w) {
+      if (w < warp) at += bytes_of[w], k += kept_of[w];
+      n_bytes += bytes_of[w], n_out += kept_of[w];
+    }
+    if (keep) {
+      if (filter) kept[k] = m;
+      if (ebase) ebase[k] = at;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    if (filter) *n_kept = n_out;
+    if (ebase) ebase[n_out] = ebase[cap] = n_bytes;
+  }
+}
+
 // qualities of field 0 (the amplicon or its trimmed interior) at the field's arena offset, reversed
 // for RF like the bases (qualities are not complemented); one warp per amplicon
 __global__ void k_extract_qual(const ah_amplicon* __restrict__ amps, uint64_t n, const ah_hit* __restrict__ hits,
@@ -216,6 +271,13 @@ __global__ void k_extract_qual(const ah_amplicon* __restrict__ amps, uint64_t n,
 }
 
 }  // namespace
+
+void launch_finish_one(cudaStream_t s, ah_amplicon* amps, uint64_t cap, const uint64_t* d_n, const double* hit_tm,
+                       int filter, double min_tm, ah_amplicon* kept, uint64_t* n_kept, const ah_hit* hits,
+                       const uint32_t* rec_len, const uint8_t* plen, int trim, uint32_t fb, uint32_t rb, uint64_t* ebase) {
+  k_finish_one<<<1, kOneThreads, 0, s>>>(amps, cap, d_n, hit_tm, filter, min_tm, kept, n_kept, hits, rec_len, plen, trim,
+                                         (int64_t)fb, (int64_t)rb, ebase);
+}
 
 void launch_extract(cudaStream_t s, bool write, const ah_amplicon* amps, uint64_t cap, const uint64_t* d_n,
                     const ah_hit* hits, const uint2* planes, const uint32_t* invalid, const uint64_t* rec_group,
@@ -246,9 +308,9 @@ ah_status extract(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const ah_
     k_extract_len<<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(a->d, n, h->d, b->rec_len, p->d_plen, trim,
                                                                        (int64_t)fb, (int64_t)rb, tot);
   if (n) launched(ctx);
-  if ((st = exclusive_scan_u64(ctx, tot, base, n))) return st;
-  uint64_t bytes = 0;
-  if ((st = read_u64(ctx, base + n, &bytes))) return st;
+  if ((st = exclusive_scan_u64(ctx, tot, base, n, ctx->h_read))) return st;
+  AH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  const uint64_t bytes = ctx->h_read[0];
   if ((st = dalloc(ctx, &a->d_arena, bytes)) || (st = dalloc(ctx, &a->d_field_off, 5 * n + 1))) return st;
   if (n) {
     k_extract_write<<<extract_blocks(n), kExThreads, 0, ctx->stream>>>(a->d, n, h->d, b->planes, b->invalid, b->rec_group,

@@ -247,8 +247,9 @@ ah_status dalloc(ah_ctx* ctx, T** p, size_t count) {
 void dfree(ah_ctx* ctx, void* p);
 
 // ---- exclusive scan over counts: out[i] = sum(in[0..i)), out[n] = total ------------------------
-ah_status exclusive_scan_u32(ah_ctx* ctx, const uint32_t* d_in, uint64_t* d_out, uint64_t n);
-ah_status exclusive_scan_u64(ah_ctx* ctx, const uint64_t* d_in, uint64_t* d_out, uint64_t n);
+// (host: page-locked, gets the total too once the stream has passed the scan)
+ah_status exclusive_scan_u32(ah_ctx* ctx, const uint32_t* d_in, uint64_t* d_out, uint64_t n, uint64_t* host = nullptr);
+ah_status exclusive_scan_u64(ah_ctx* ctx, const uint64_t* d_in, uint64_t* d_out, uint64_t n, uint64_t* host = nullptr);
 // device -> host copy into caller memory, synchronous: page-locked destinations directly, pageable
 // ones through the context's two page-locked bounce buffers, so that no copy takes the driver's
 // pageable path (one staging pipeline for every stream of the process)
@@ -390,7 +391,21 @@ ah_status tm_tab_image(ah_ctx* ctx, int slot, const int32_t** out);
 void launch_tm(cudaStream_t s, const void* run, const ah_hit* hits, uint64_t hit_cap, const uint64_t* d_nhits,
                const ah_primers* p, uint32_t* status, const uint2* planes, const uint64_t* rec_group, double* hit_tm,
                ah_amplicon* amps, uint64_t amp_cap, const uint64_t* d_namps, int filter, double min_tm, uint32_t* keep,
-               uint32_t* defer, int sm_count, const TmKernel& tk);
+               uint32_t* defer, int sm_count, const TmKernel& tk,
+               bool marked = false, bool sites_only = false);
+// Plans with few sites and amplicons: the pairing (both walks, the scan between them, the marking of the sites whose
+// Tm is wanted) and what follows the Tm stage up to the extraction (threshold, compaction, lengths, their scan) in one
+// block each.  total: the amplicons found; ebase (may be null): offsets of the kept amplicons' bytes and their total.
+// (A replay with 64 sites takes 53 us this way and 69 over many blocks, with 2,048 sites 96 and 105, with 4,096 110 and
+// 108; a plan that sizes its own buffers at 4,096 holds up to 2,457.)
+constexpr uint64_t kOneBlockItems = 4096;
+constexpr unsigned long long kWantedMark = 0xFFFFFFFFFFFFFFFFull;  // the Tm kernels' kSiteWanted
+void launch_pairs_one(cudaStream_t s, const ah_hit* hits, uint64_t cap, const uint64_t* d_n, const uint64_t* pair_off,
+                      const uint8_t* plen, uint32_t min_len, uint32_t max_len, uint32_t mask, ah_amplicon* out,
+                      uint64_t out_cap, uint32_t* overflow, double* hit_tm, uint64_t* total);
+void launch_finish_one(cudaStream_t s, ah_amplicon* amps, uint64_t cap, const uint64_t* d_n, const double* hit_tm,
+                       int filter, double min_tm, ah_amplicon* kept, uint64_t* n_kept, const ah_hit* hits,
+                       const uint32_t* rec_len, const uint8_t* plen, int trim, uint32_t fb, uint32_t rb, uint64_t* ebase);
 void launch_compact_amps(cudaStream_t s, const ah_amplicon* in, uint64_t cap, const uint32_t* keep, const uint64_t* off,
                          ah_amplicon* out);
 void launch_extract(cudaStream_t s, bool write, const ah_amplicon* amps, uint64_t cap, const uint64_t* d_n,

@@ -14,16 +14,14 @@ __device__ __forceinline__ uint8_t orientation(uint32_t primer_i, uint32_t prime
   return (uint8_t)(primer_i == primer_j ? 2u + primer_i : primer_i);
 }
 
-// d_n (optional): live site count in device memory, n is then the capacity; out_cap and overflow
-// (optional) bound the emitted records
+// Site i's walk, by whole warps.  Counting: the number of its partners; emitting: their amplicons from out[w] on as far
+// as out_cap goes (past it the overflow bit), with both sites marked in hit_tm (may be null) as wanted.
 template <bool kEmit>
-__global__ void k_pair_walk(const ah_hit* __restrict__ hits, uint64_t n, const uint64_t* __restrict__ pair_off,
-                            const uint8_t* __restrict__ plen, uint32_t min_len, uint32_t max_len, uint32_t mask,
-                            uint32_t* __restrict__ counts, const uint64_t* __restrict__ out_off,
-                            ah_amplicon* __restrict__ out, const uint64_t* __restrict__ d_n = nullptr,
-                            uint64_t out_cap = ~0ull, uint32_t* __restrict__ overflow = nullptr) {
-  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t n_live = d_n ? min(*d_n, n) : n;
+__device__ __forceinline__ uint32_t pair_walk(const ah_hit* __restrict__ hits, uint64_t i, uint64_t n_live,
+                                              const uint64_t* __restrict__ pair_off, const uint8_t* __restrict__ plen,
+                                              uint32_t min_len, uint32_t max_len, uint32_t mask, uint64_t w,
+                                              ah_amplicon* __restrict__ out, uint64_t out_cap,
+                                              uint32_t* __restrict__ overflow, unsigned long long* __restrict__ hit_tm) {
   const uint32_t lane = threadIdx.x & 31u;
   const bool live = i < n_live;
   ah_hit a{};
@@ -33,7 +31,6 @@ __global__ void k_pair_walk(const ah_hit* __restrict__ hits, uint64_t n, const u
   const uint32_t pair = a.pattern >> 2;
   const uint64_t seg_end = walking ? min(pair_off[pair + 1], n_live) : 0;
   uint32_t cnt = 0;
-  uint64_t w = kEmit && live ? out_off[i] : 0;
   // partner j of the anchor: false when the walk ends there
   auto partner = [&](uint64_t j, uint32_t b_record, uint32_t b_pos, uint32_t b_pattern) -> bool {
     if (b_record != a.record) return false;
@@ -56,10 +53,12 @@ __global__ void k_pair_walk(const ah_hit* __restrict__ hits, uint64_t n, const u
       m.orient = o;
       m.flags = 0;
       m.tm = __longlong_as_double(0x7ff8000000000000ll);
-      if (w < out_cap)
+      if (w < out_cap) {
         out[w] = m;
-      else if (overflow)
+        if (hit_tm) hit_tm[i] = hit_tm[j] = kWantedMark;
+      } else if (overflow) {
         atomicOr(overflow, 4u);
+      }
       ++w;
     } else {
       ++cnt;
@@ -84,7 +83,62 @@ __global__ void k_pair_walk(const ah_hit* __restrict__ hits, uint64_t n, const u
     const ah_hit b = hits[j];
     walking = partner(j, b.record, b.pos, b.pattern);
   }
+  return cnt;
+}
+
+// d_n (optional): live site count in device memory, n is then the capacity; out_cap and overflow
+// (optional) bound the emitted records
+template <bool kEmit>
+__global__ void k_pair_walk(const ah_hit* __restrict__ hits, uint64_t n, const uint64_t* __restrict__ pair_off,
+                            const uint8_t* __restrict__ plen, uint32_t min_len, uint32_t max_len, uint32_t mask,
+                            uint32_t* __restrict__ counts, const uint64_t* __restrict__ out_off,
+                            ah_amplicon* __restrict__ out, const uint64_t* __restrict__ d_n = nullptr,
+                            uint64_t out_cap = ~0ull, uint32_t* __restrict__ overflow = nullptr) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t n_live = d_n ? min(*d_n, n) : n;
+  const uint32_t cnt = pair_walk<kEmit>(hits, i, n_live, pair_off, plen, min_len, max_len, mask,
+                                        kEmit && i < n_live ? out_off[i] : 0, out, out_cap, overflow, nullptr);
   if (!kEmit && i < n) counts[i] = cnt;
+}
+
+// The whole stage in one block for up to kOneBlockItems sites: 1,024 sites at a time are counted, scanned and walked
+// again; hit_tm is cleared and the amplicons' sites marked for the Tm stage.  A launch and its gap cost more than such
+// a walk: 75 sites took 21 us in six kernels, 6.8 here.
+constexpr int kOneThreads = 1024;
+__global__ void __launch_bounds__(kOneThreads) k_pairs_one(
+    const ah_hit* __restrict__ hits, uint64_t cap, const uint64_t* __restrict__ d_n, const uint64_t* __restrict__ pair_off,
+    const uint8_t* __restrict__ plen, uint32_t min_len, uint32_t max_len, uint32_t mask, ah_amplicon* __restrict__ out,
+    uint64_t out_cap, uint32_t* __restrict__ overflow, unsigned long long* __restrict__ hit_tm,
+    uint64_t* __restrict__ total) {
+  __shared__ uint32_t sums[kOneThreads / 32];
+  const uint64_t n = min(*d_n, cap);
+  for (uint64_t i = threadIdx.x; i < cap; i += kOneThreads) hit_tm[i] = 0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint64_t carry = 0;
+  for (uint64_t base = 0; base < n; base += kOneThreads) {
+    const uint64_t i = base + threadIdx.x;
+    const uint32_t cnt = pair_walk<false>(hits, i, n, pair_off, plen, min_len, max_len, mask, 0, nullptr, 0, nullptr, nullptr);
+    uint32_t inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) sums[warp] = inc;
+    __syncthreads();  // also the cleared marks
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < kOneThreads / 32; ++w) {
+      const uint32_t x = sums[w];
+      before += w < warp ? x : 0u;
+      all += x;
+    }
+    __syncthreads();
+    pair_walk<true>(hits, i, n, pair_off, plen, min_len, max_len, mask, carry + before + inc - cnt, out, out_cap, overflow,
+                    hit_tm);
+    carry += all;
+  }
+  if (threadIdx.x == 0) *total = carry;
 }
 
 }  // namespace
@@ -102,6 +156,13 @@ void launch_pair_walk(cudaStream_t s, bool emit, const ah_hit* hits, uint64_t ca
                                               nullptr, d_n, out_cap, overflow);
 }
 
+void launch_pairs_one(cudaStream_t s, const ah_hit* hits, uint64_t cap, const uint64_t* d_n, const uint64_t* pair_off,
+                      const uint8_t* plen, uint32_t min_len, uint32_t max_len, uint32_t mask, ah_amplicon* out,
+                      uint64_t out_cap, uint32_t* overflow, double* hit_tm, uint64_t* total) {
+  k_pairs_one<<<1, kOneThreads, 0, s>>>(hits, cap, d_n, pair_off, plen, min_len, max_len, mask, out, out_cap, overflow,
+                                        reinterpret_cast<unsigned long long*>(hit_tm), total);
+}
+
 ah_status pair_amplicons(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const ah_hits* h, uint32_t min_len,
                          uint32_t max_len, uint32_t orient_mask, ah_amplicons** out) {
   (void)b;
@@ -117,9 +178,9 @@ ah_status pair_amplicons(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
                                                         orient_mask, counts, nullptr, nullptr);
     launched(ctx);
   }
-  if ((st = exclusive_scan_u32(ctx, counts, off, n))) return st;
-  uint64_t total = 0;
-  if ((st = read_u64(ctx, off + n, &total))) return st;
+  if ((st = exclusive_scan_u32(ctx, counts, off, n, ctx->h_read))) return st;
+  AH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  const uint64_t total = ctx->h_read[0];
   if (total > 0xffffffffull) return fail(ctx, AH_EOVERFLOW, "pairing: more than 2^32 amplicons");
   ah_amplicons* a = new ah_amplicons();
   a->ctx = ctx;

@@ -134,6 +134,18 @@ void enqueue_step(ah_plan* pl, cudaStream_t s) {
   enqueue_post(pl, s);
 }
 
+// The counters of a run and the status word to page-locked memory, where ah_plan_check finds them after one wait
+// (five copies and a second round trip for the status before).
+__global__ void k_plan_summary(const uint32_t* ctr, const uint64_t* n_hits, const uint64_t* n_amps, const uint64_t* n_kept,
+                               const uint64_t* arena_bytes, const uint32_t* status, uint64_t* out) {
+  out[0] = ctr[0];
+  out[1] = *n_hits;
+  out[2] = *n_amps;
+  if (n_kept) out[3] = *n_kept;
+  if (arena_bytes) out[4] = *arena_bytes;
+  out[5] = *status;
+}
+
 void enqueue_post(ah_plan* pl, cudaStream_t s) {
   const ah_batch* b = pl->b;
   const ah_primers* p = pl->p;
@@ -145,31 +157,46 @@ void enqueue_post(ah_plan* pl, cudaStream_t s) {
   launch_emit_hits(s, pl->slots, pl->tile_count, pl->slot_cap, pl->n_tiles, pl->tile_groups, pl->tpc_off, b, pl->hits,
                    nullptr, pl->hit_cap, pl->ctr + 1, pl->pair_off, p->n_pairs);
   const uint64_t* n_hits = pl->tpc_off + pl->n_cells;
-  launch_pair_walk(s, false, pl->hits, pl->hit_cap, n_hits, pl->pair_off, p->d_plen, q.min_len, q.max_len,
-                   q.orient_mask & 15u, pl->pcount, nullptr, nullptr, 0, nullptr);
-  exclusive_scan_u32_s(s, pl->pcount, pl->poff, pl->hit_cap, pl->scratch);
-  launch_pair_walk(s, true, pl->hits, pl->hit_cap, n_hits, pl->pair_off, p->d_plen, q.min_len, q.max_len,
-                   q.orient_mask & 15u, nullptr, pl->poff, pl->amps, pl->amp_cap, pl->ctr + 1);
-  const uint64_t* n_amps = pl->poff + pl->hit_cap;
+  // few sites and amplicons: one block each for the pairing and for what follows the Tm stage
+  const bool few_hits = pl->hit_cap <= kOneBlockItems, few_amps = pl->amp_cap <= kOneBlockItems;
+  uint64_t* n_amps = pl->poff + pl->hit_cap;
+  if (few_hits) {
+    launch_pairs_one(s, pl->hits, pl->hit_cap, n_hits, pl->pair_off, p->d_plen, q.min_len, q.max_len, q.orient_mask & 15u,
+                     pl->amps, pl->amp_cap, pl->ctr + 1, pl->hit_tm, n_amps);
+  } else {
+    launch_pair_walk(s, false, pl->hits, pl->hit_cap, n_hits, pl->pair_off, p->d_plen, q.min_len, q.max_len,
+                     q.orient_mask & 15u, pl->pcount, nullptr, nullptr, 0, nullptr);
+    exclusive_scan_u32_s(s, pl->pcount, pl->poff, pl->hit_cap, pl->scratch);
+    launch_pair_walk(s, true, pl->hits, pl->hit_cap, n_hits, pl->pair_off, p->d_plen, q.min_len, q.max_len,
+                     q.orient_mask & 15u, nullptr, pl->poff, pl->amps, pl->amp_cap, pl->ctr + 1);
+  }
   launch_tm(s, pl->tm_run, pl->hits, pl->hit_cap, n_hits, p, pl->ctx->d_status, b->planes, b->rec_group, pl->hit_tm,
             pl->amps, pl->amp_cap, n_amps, q.tm.filter, q.tm.min_tm, pl->keep, pl->tm_defer, pl->ctx->sm_count,
-            pl->tm_k);
+            pl->tm_k, few_hits, few_amps);
   const ah_amplicon* out = pl->amps;
   const uint64_t* n_out = n_amps;
-  if (q.tm.filter) {
+  if (few_amps) {
+    launch_finish_one(s, pl->amps, pl->amp_cap, n_amps, pl->hit_tm, q.tm.filter, q.tm.min_tm, pl->kept,
+                      pl->koff + pl->amp_cap, pl->hits, b->rec_len, p->d_plen, q.trim, q.fb_len, q.rb_len,
+                      q.extract ? pl->ebase : nullptr);
+    if (q.tm.filter) out = pl->kept, n_out = pl->koff + pl->amp_cap;
+  } else if (q.tm.filter) {
     exclusive_scan_u32_s(s, pl->keep, pl->koff, pl->amp_cap, pl->scratch);
     launch_compact_amps(s, pl->amps, pl->amp_cap, pl->keep, pl->koff, pl->kept);
     out = pl->kept;
     n_out = pl->koff + pl->amp_cap;
   }
-  if (q.extract) {
+  if (q.extract && !few_amps) {
     launch_extract(s, false, out, pl->amp_cap, n_out, pl->hits, b->planes, b->invalid, b->rec_group, b->rec_len,
                    p->d_plen, q.trim, q.fb_len, q.rb_len, pl->elen, nullptr, nullptr, 0, nullptr);
     exclusive_scan_u64_s(s, pl->elen, pl->ebase, pl->amp_cap, pl->scratch);
+  }
+  k_plan_summary<<<1, 1, 0, s>>>(pl->ctr, n_hits, n_amps, q.tm.filter ? n_out : nullptr,
+                                 q.extract ? pl->ebase + pl->amp_cap : nullptr, pl->ctx->d_status, pl->h_out);
+  if (q.extract)
     launch_extract(s, true, out, pl->amp_cap, n_out, pl->hits, b->planes, b->invalid, b->rec_group, b->rec_len,
                    p->d_plen, q.trim, q.fb_len, q.rb_len, pl->ebase, pl->arena, pl->field_off, pl->arena_cap,
                    pl->ctr + 1);
-  }
 }
 
 ah_status capture(ah_plan* pl) {
@@ -418,6 +445,7 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
   }
   if (!st && cudaMallocHost(&pl->h_out, 8 * sizeof(uint64_t)) != cudaSuccess)
     st = fail(ctx, AH_ENOMEM, "ah_plan_create: pinned allocation failed");
+  if (!st) std::fill(pl->h_out, pl->h_out + 8, 0);
   if (!st) st = alloc_buffers(pl);
   if (!st) st = capture(pl);
   // checked replays: the per-tile slot lists (sized from the context's default) and the capacities
@@ -673,18 +701,10 @@ ah_status ah_plan_check(ah_plan* pl) {
   if (!pl) return AH_EINVAL;
   ah_ctx* c = pl->ctx;
   cudaStream_t s = c->stream;
-  AH_CUDA(c, cudaMemcpyAsync(pl->h_out + 0, pl->ctr, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  AH_CUDA(c, cudaMemcpyAsync(pl->h_out + 1, pl->tpc_off + pl->n_cells, 8, cudaMemcpyDeviceToHost, s));
-  AH_CUDA(c, cudaMemcpyAsync(pl->h_out + 2, pl->poff + pl->hit_cap, 8, cudaMemcpyDeviceToHost, s));
-  if (pl->prm.tm.filter)
-    AH_CUDA(c, cudaMemcpyAsync(pl->h_out + 3, pl->koff + pl->amp_cap, 8, cudaMemcpyDeviceToHost, s));
-  if (pl->prm.extract)
-    AH_CUDA(c, cudaMemcpyAsync(pl->h_out + 4, pl->ebase + pl->amp_cap, 8, cudaMemcpyDeviceToHost, s));
   AH_CUDA(c, cudaStreamSynchronize(s));
-  ah_status st = check_status(c);
-  if (st) return st;
-  const uint32_t* cw = (const uint32_t*)pl->h_out;
-  const uint32_t max_tile = cw[0];
+  ah_status st;
+  if (pl->h_out[5] && (st = check_status(c))) return st;
+  const uint32_t max_tile = (uint32_t)pl->h_out[0];
   pl->info.n_hits = pl->h_out[1];
   pl->info.n_amps = pl->h_out[2];
   pl->info.n_kept = pl->prm.tm.filter ? pl->h_out[3] : std::min(pl->h_out[2], pl->amp_cap);
@@ -800,7 +820,10 @@ void ah_plan_free(ah_plan* pl) {
         break;
       }
     free_buffers(pl);
-    if (pl->h_out) cudaFreeHost(pl->h_out);
+    if (pl->h_out) {
+      cudaStreamSynchronize(pl->ctx->stream);  // a replay in flight writes it
+      cudaFreeHost(pl->h_out);
+    }
     for (cudaEvent_t e : pl->scan_ev)
       if (e) cudaEventDestroy(e);
     for (auto& pr : pl->ring_ev)

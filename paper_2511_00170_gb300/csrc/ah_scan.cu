@@ -209,8 +209,11 @@ __global__ void k_emit_hits(const uint64_t* __restrict__ slots, const uint32_t* 
                             uint64_t n_tiles, uint64_t tile_groups, const uint64_t* __restrict__ off,
                             const uint64_t* __restrict__ rec_group, uint32_t n_rec, ah_hit* __restrict__ hits,
                             const uint64_t* __restrict__ tile_base = nullptr, uint64_t hit_cap = ~0ull,
-                            uint32_t* __restrict__ overflow = nullptr) {
+                            uint32_t* __restrict__ overflow = nullptr, uint64_t* __restrict__ pair_off = nullptr,
+                            uint32_t n_pairs = 0) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (pair_off && blockIdx.x == 0)  // each pair's first hit
+    for (uint32_t p = threadIdx.x; p <= n_pairs; p += blockDim.x) pair_off[p] = off[(uint64_t)p * n_tiles];
   const uint64_t t = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (t >= n_tiles) return;
   const uint32_t n = min(tile_count[t], cap);
@@ -264,12 +267,6 @@ __global__ void k_emit_hits(const uint64_t* __restrict__ slots, const uint32_t* 
     else if (overflow)
       atomicOr(overflow, 2u);
   }
-}
-
-__global__ void k_pair_offsets(const uint64_t* __restrict__ off, uint64_t n_tiles, uint32_t n_pairs,
-                               uint64_t* __restrict__ pair_off) {
-  uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p <= n_pairs) pair_off[p] = off[(uint64_t)p * n_tiles];
 }
 
 // What the host needs before it sizes a scan's output, written straight into page-locked memory: the
@@ -500,8 +497,8 @@ void launch_emit_hits(cudaStream_t s, const uint64_t* slots, const uint32_t* til
                       const uint64_t* tile_base, uint64_t hit_cap, uint32_t* overflow, uint64_t* pair_off,
                       uint32_t n_pairs) {
   k_emit_hits<<<(unsigned)((n_tiles + 7) / 8), 256, 0, s>>>(slots, tile_count, cap, n_tiles, tile_groups, off,
-                                                            b->rec_group, b->n_records, hits, tile_base, hit_cap, overflow);
-  k_pair_offsets<<<(n_pairs + 256) / 256, 256, 0, s>>>(off, n_tiles, n_pairs, pair_off);
+                                                            b->rec_group, b->n_records, hits, tile_base, hit_cap, overflow,
+                                                            pair_off, n_pairs);
 }
 
 namespace {

@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "ah_amps.cuh"
 #include "ah_internal.h"
 
 namespace ah {
@@ -1058,6 +1059,7 @@ __device__ double group_site_tm(TmGroupSh& sh, int32_t* w, int L, int k, int cla
 // sites'): the amplicons first write kSiteWanted into hit_tm at their two sites, over an array
 // cleared to zero, and the Tm kernels take only the marked sites.
 
+static_assert(kWantedMark == kSiteWanted, "the pairing marks sites for the Tm kernels");
 __global__ void k_mark_sites(const ah_amplicon* __restrict__ a, uint64_t n, double* __restrict__ hit_tm,
                              const uint64_t* __restrict__ d_n = nullptr) {
   const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1729,19 +1731,7 @@ __global__ void k_tm_amps(ah_amplicon* __restrict__ a, uint64_t n, const double*
     return;
   }
   ah_amplicon m = a[i];
-  const double ti = hit_tm[m.hit_i], tj = hit_tm[m.hit_j];
-  const bool undefined = isnan(ti) || isnan(tj);
-  const double t = undefined ? __longlong_as_double(0x7ff8000000000000ll) : fmin(ti, tj);
-  // bit0: the threshold decision (defined and Tm >= min_tm), bit1: Tm within 1e-9 C of min_tm, so
-  // that the decision rests on the last digits of a double, bit2: undefined.  Without the filter
-  // the list is not compacted and the bits only annotate.
-  const bool pass = !undefined && t >= min_tm;
-  uint8_t flags = 0;
-  if (pass) flags |= 1;
-  if (!undefined && fabs(t - min_tm) <= 1e-9) flags |= 2;
-  if (undefined) flags |= 4;
-  m.tm = t;
-  m.flags = flags;
+  const bool pass = decide_amplicon(&m, hit_tm[m.hit_i], hit_tm[m.hit_j], min_tm);
   a[i] = m;
   if (keep) keep[i] = (!filter || pass) ? 1u : 0u;
 }
@@ -2040,11 +2030,14 @@ ah_status tm_prepare(ah_ctx* ctx, const ah_tm_params* params, void* run_out, siz
 void launch_tm(cudaStream_t s, const void* run, const ah_hit* hits, uint64_t hit_cap, const uint64_t* d_nhits,
                const ah_primers* p, uint32_t* status, const uint2* planes, const uint64_t* rec_group, double* hit_tm,
                ah_amplicon* amps, uint64_t amp_cap, const uint64_t* d_namps, int filter, double min_tm, uint32_t* keep,
-               uint32_t* defer, int sm_count, const TmKernel& tk) {
+               uint32_t* defer, int sm_count, const TmKernel& tk, bool marked, bool sites_only) {
   const TmRun R = *(const TmRun*)run;
-  cudaMemsetAsync(hit_tm, 0, std::max<uint64_t>(1, hit_cap) * sizeof(double), s);
-  k_mark_sites<<<(unsigned)std::max<uint64_t>(1, (amp_cap + 255) / 256), 256, 0, s>>>(amps, amp_cap, hit_tm, d_namps);
+  if (!marked) {
+    cudaMemsetAsync(hit_tm, 0, std::max<uint64_t>(1, hit_cap) * sizeof(double), s);
+    k_mark_sites<<<(unsigned)std::max<uint64_t>(1, (amp_cap + 255) / 256), 256, 0, s>>>(amps, amp_cap, hit_tm, d_namps);
+  }
   launch_tm_hits(s, R, p, hits, hit_cap, d_nhits, planes, rec_group, hit_tm, status, defer, sm_count, tk, nullptr);
+  if (sites_only) return;
   k_tm_amps<<<(unsigned)std::max<uint64_t>(1, (amp_cap + 255) / 256), 256, 0, s>>>(amps, amp_cap, hit_tm, filter,
                                                                                   min_tm, keep, d_namps);
 }
@@ -2087,11 +2080,11 @@ ah_status tm_filter(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const a
   if (params->filter) {
     uint64_t* off;
     if ((st = dalloc(ctx, &off, a->n + 1))) return st;
-    if ((st = exclusive_scan_u32(ctx, keep, off, a->n))) return st;
+    if ((st = exclusive_scan_u32(ctx, keep, off, a->n, ctx->h_read))) return st;
     // the number kept and the status word in one round trip
     AH_CUDA(ctx, cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
-    uint64_t kept = 0;
-    if ((st = read_u64(ctx, off + a->n, &kept))) return st;
+    AH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    const uint64_t kept = ctx->h_read[0];
     const bool flagged = *ctx->h_status != 0;
     ah_amplicon* nd = nullptr;
     if ((st = dalloc(ctx, &nd, kept))) return st;
