@@ -1646,8 +1646,8 @@ __global__ void __launch_bounds__(kTmThreads, 4) k_tm_hits_t(const ah_hit* __res
                                                              const uint8_t* __restrict__ plen,
                                                              const uint4* __restrict__ pmask, const TmRun Rp,
                                                              double* __restrict__ out, uint32_t* __restrict__ defer,
-                                                             const uint64_t* __restrict__ d_n) {
-  tm_hits_body<GenericSites>(hits, n, planes, rec_group, plen, pmask, Rp, out, defer, d_n, nullptr, 0u, ~0u);
+                                                             const uint64_t* __restrict__ d_n, int window) {
+  tm_hits_body<GenericSites>(hits, n, planes, rec_group, plen, pmask, Rp, out, defer, d_n, nullptr, 0u, ~0u, window);
 }
 
 // The sites k_tm_hits_t listed (defer[0] of them at defer[1..]): one warp per site, every lane
@@ -1855,7 +1855,12 @@ int launch_tm_hits(cudaStream_t s, const TmRun& R, const ah_primers* p, const ah
   int n_launched = 0;
   if (const size_t smem = thread_kernel_smem(p, R.variants)) {
     cudaMemsetAsync(defer, 0, sizeof(uint32_t), s);
-    const unsigned grid = (unsigned)std::max<uint64_t>(1, (cap + kTmSlots - 1) / kTmSlots);
+    // fewer sites: smaller windows, down to one site per thread, until sixteen blocks per SM have work (a thread takes
+    // its share of a window's sites one after another, a chain of some 12 us each).  344,000 slots of reads 75 -> 43 us
+    // (four blocks per SM: 50), 38,000 slots 58 -> 18, 11,000 slots of eight pairs 69 -> 26; below 128 slots nothing more.
+    int window = kTmSlots;
+    while (window > kTmThreads && cap < 16ull * (uint64_t)std::max(1, sm_count) * (uint64_t)window) window /= 2;
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, (cap + window - 1) / window);
     const size_t smem_j = 4 * ((size_t)kTmThreadFixedWords + (size_t)tk.weight_words * kTmThreads);
     if (tk.fn && tk.image && smem_j <= kTmSmemCap) {  // the kernel generated for this primer set
       const uint8_t* plen = p->d_plen;
@@ -1868,14 +1873,14 @@ int launch_tm_hits(cudaStream_t s, const TmRun& R, const ah_primers* p, const ah
         uint32_t pr_lo = parts > 1 ? n_pr * k / parts : 0u, pr_hi = parts > 1 ? n_pr * (k + 1) / parts : ~0u;
         void* args[] = {(void*)&hits, (void*)&cap,    (void*)&planes, (void*)&rec_group, (void*)&plen, (void*)&pmask,
                         (void*)&R,    (void*)&hit_tm, (void*)&defer,  (void*)&d_n,       (void*)&tk.image,
-                        (void*)&pr_lo, (void*)&pr_hi};
+                        (void*)&pr_lo, (void*)&pr_hi,  (void*)&window};
         cudaLaunchKernel((const void*)tk.fn, dim3(grid), dim3(kTmThreads), args, smem_j, s);
       }
       if (generated) *generated = true;
       n_launched += parts;
     } else {
       k_tm_hits_t<<<grid, kTmThreads, smem, s>>>(hits, cap, planes, rec_group, p->d_plen, p->d_pmask, R, hit_tm, defer,
-                                                 d_n);
+                                                 d_n, window);
       ++n_launched;
     }
     const size_t smem_d = smem - 4 * (size_t)(2 * kTmSlots);  // tables and weights only

@@ -215,7 +215,7 @@ __device__ __forceinline__ bool chain_site_tm(const TmTabs& T, int32_t* __restri
 }
 
 // The site Tm of every marked site of a launch.  Blocks of kTmThreads threads take windows of
-// kTmSlots site slots.  Each thread first settles its slots where that needs no chain (not wanted,
+// `window` site slots (kTmSlots at most).  Each thread first settles its slots where that needs no chain (not wanted,
 // or a step between two single-choice positions without a parameter: every variant contains it,
 // NaN); the rest are sorted by primer and taken in that order, kTmThreads at a time, so the threads
 // of a warp share the chain's shape and the warps are full.  Sites the chain does not cover go to
@@ -230,7 +230,7 @@ __device__ __forceinline__ void tm_hits_body(const ah_hit* __restrict__ hits, ui
                                              const uint8_t* __restrict__ plen, const uint4* __restrict__ pmask,
                                              const TmRun& Rp, double* __restrict__ out, uint32_t* __restrict__ defer,
                                              const uint64_t* __restrict__ d_n, const int32_t* __restrict__ image,
-                                             uint32_t pr_lo, uint32_t pr_hi) {
+                                             uint32_t pr_lo, uint32_t pr_hi, int window) {
   // the run constants in shared memory: device functions take them by reference, and a reference
   // to a kernel parameter would make the compiler copy it to local memory for every thread
   __shared__ TmRun R_sh;
@@ -246,10 +246,10 @@ __device__ __forceinline__ void tm_hits_body(const ah_hit* __restrict__ hits, ui
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
   D::fill(T, image, Rp.nn);
   __syncthreads();
-  const uint64_t base = (uint64_t)blockIdx.x * kTmSlots;
+  const uint64_t base = (uint64_t)blockIdx.x * (uint64_t)window;
   const uint64_t n_here = d_n && *d_n < n ? *d_n : n;
   int mine = 0;
-  for (int t = threadIdx.x; t < kTmSlots; t += kTmThreads) {
+  for (int t = threadIdx.x; t < window; t += kTmThreads) {
     const uint64_t i = base + t;
     uint32_t key = 0xFFFFFFFFu;
     if (i < n_here && (unsigned long long)__double_as_longlong(out[i]) == kSiteWanted) {
@@ -286,7 +286,7 @@ __device__ __forceinline__ void tm_hits_body(const ah_hit* __restrict__ hits, ui
   // bins, which can only mix shapes, never lose a site); order within a primer does not matter
   for (int k = threadIdx.x; k < kTmBins; k += kTmThreads) bins[k] = 0;
   __syncthreads();
-  for (int t = threadIdx.x; t < kTmSlots; t += kTmThreads)
+  for (int t = threadIdx.x; t < window; t += kTmThreads)
     if (keys[t] != 0xFFFFFFFFu) atomicAdd(&bins[(keys[t] >> 16) % kTmBins], 1u);
   __syncthreads();
   if (threadIdx.x < 32) {  // exclusive scan of the bins, kTmBins / 32 per lane
@@ -302,7 +302,7 @@ __device__ __forceinline__ void tm_hits_body(const ah_hit* __restrict__ hits, ui
     for (int k = 0; k < per; ++k) bins[threadIdx.x * per + k] = run, run += v[k];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < kTmSlots; t += kTmThreads) {
+  for (int t = threadIdx.x; t < window; t += kTmThreads) {
     const uint32_t key = keys[t];
     if (key != 0xFFFFFFFFu) order[atomicAdd(&bins[(key >> 16) % kTmBins], 1u)] = key;
   }

@@ -371,8 +371,9 @@ std::string tm_chain_source(const std::vector<std::string>& primers, int* weight
         "    const ah_hit* __restrict__ hits, uint64_t n, const uint2* __restrict__ planes,\n"
         "    const uint64_t* __restrict__ rec_group, const uint8_t* __restrict__ plen, const uint4* __restrict__ pmask,\n"
         "    const TmRun Rp, double* __restrict__ out, uint32_t* __restrict__ defer, const uint64_t* __restrict__ d_n,\n"
-        "    const int32_t* __restrict__ image, uint32_t pr_lo, uint32_t pr_hi) {\n"
-        "  tm_hits_body<GenSites>(hits, n, planes, rec_group, plen, pmask, Rp, out, defer, d_n, image, pr_lo, pr_hi);\n}\n";
+        "    const int32_t* __restrict__ image, uint32_t pr_lo, uint32_t pr_hi, int window) {\n"
+        "  tm_hits_body<GenSites>(hits, n, planes, rec_group, plen, pmask, Rp, out, defer, d_n, image, pr_lo, pr_hi,\n"
+        "                         window);\n}\n";
   if (weight_words) *weight_words = words;
   return os.str();
 }
