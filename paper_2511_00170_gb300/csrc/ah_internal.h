@@ -350,11 +350,10 @@ void launch_scan_kernel(cudaStream_t s, const ScanKernel& k, const ah_batch* b, 
 // a one-CTA-per-tile kernel over groups [g0, g1) of b (g0 a multiple of the tile, g1 of it or the end)
 void launch_scan_range(cudaStream_t s, const ScanKernel& k, const ah_batch* b, uint64_t* slots, uint32_t* tile_count,
                        uint32_t cap, uint32_t* status, uint64_t g0, uint64_t g1);
-void launch_tile_max(cudaStream_t s, const uint32_t* tile_count, uint64_t n_tiles, uint32_t* out);
 // sorts every tile's keys and counts them per pair; big: n_tiles + 1 words of device scratch, used
 // when cap exceeds 256; returns the kernels launched
 int launch_tile_sort(cudaStream_t s, uint64_t* slots, const uint32_t* tile_count, uint32_t cap, uint64_t n_tiles,
-                     uint32_t n_pairs, uint32_t* tpc, uint32_t* big, int sm_count);
+                     uint32_t n_pairs, uint32_t* tpc, uint32_t* big, int sm_count, uint32_t* fullest);
 void launch_emit_hits(cudaStream_t s, const uint64_t* slots, const uint32_t* tile_count, uint32_t cap, uint64_t n_tiles,
                       uint64_t tile_groups, const uint64_t* off, const ah_batch* b, ah_hit* hits,
                       const uint64_t* tile_base, uint64_t hit_cap, uint32_t* overflow, uint64_t* pair_off,

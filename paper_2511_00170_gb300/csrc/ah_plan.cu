@@ -150,9 +150,8 @@ void enqueue_post(ah_plan* pl, cudaStream_t s) {
   const ah_batch* b = pl->b;
   const ah_primers* p = pl->p;
   const ah_plan_params& q = pl->prm;
-  launch_tile_max(s, pl->tile_count, pl->n_tiles, pl->ctr + 0);
   launch_tile_sort(s, pl->slots, pl->tile_count, pl->slot_cap, pl->n_tiles, p->n_pairs, pl->tpc, pl->big,
-                   pl->ctx->sm_count);
+                   pl->ctx->sm_count, pl->ctr + 0);
   exclusive_scan_u32_s(s, pl->tpc, pl->tpc_off, pl->n_cells, pl->scratch);
   launch_emit_hits(s, pl->slots, pl->tile_count, pl->slot_cap, pl->n_tiles, pl->tile_groups, pl->tpc_off, b, pl->hits,
                    nullptr, pl->hit_cap, pl->ctr + 1, pl->pair_off, p->n_pairs);

@@ -32,15 +32,6 @@ struct ScanParamsHost {
   uint64_t n_blocks;         // persistent kernels: blocks of threads * groups_per_thread groups
 };
 
-__global__ void k_tile_max(const uint32_t* __restrict__ tile_count, uint64_t n_tiles, uint32_t* __restrict__ out) {
-  uint32_t m = 0;
-  for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < n_tiles; t += (uint64_t)gridDim.x * blockDim.x)
-    m = max(m, tile_count[t]);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
-}
-
 __device__ __forceinline__ uint32_t lower_bound_u64(const uint64_t* a, uint32_t n, uint64_t key) {
   uint32_t lo = 0, hi = n;
   while (lo < hi) {
@@ -140,21 +131,34 @@ __device__ __forceinline__ void sort_tile(uint64_t* tk, uint32_t n, uint64_t t, 
 
 constexpr uint32_t kSmallTile = 256;  // keys a tile may hold to be sorted by one warp in registers
 
-// One warp per tile.  Tiles holding more keys are appended to big[1..] (count in big[0]) for
-// k_tile_sort_big.
+// Tiles per warp of the sort and the emission: most tiles of a large batch hold no site, and a warp each only to see
+// that took longer than the work (7.6 Gbp in 232,000 tiles, 29,500 sites: 30 us each, with eight 13 and 24); fewer tiles
+// keep a warp each, so that full ones are spread.
+inline uint32_t tiles_per_warp(uint64_t n_tiles) { return n_tiles >= 65536 ? 8u : 1u; }
+
+// A warp takes `per` tiles, one after another.  Tiles holding more keys are appended to big[1..] (count in big[0]) for
+// k_tile_sort_big.  *fullest (zero before) becomes the largest count.
 __global__ void k_tile_sort(uint64_t* __restrict__ slots, const uint32_t* __restrict__ tile_count, uint32_t cap,
                             uint64_t n_tiles, uint32_t n_pairs, uint32_t* __restrict__ tile_pair_count,
-                            uint32_t* __restrict__ big) {
+                            uint32_t* __restrict__ big, uint32_t per, uint32_t* fullest) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint64_t t = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-  if (t >= n_tiles) return;
-  const uint32_t n = min(tile_count[t], cap);
-  if (n == 0) return;
-  if (n > kSmallTile) {
-    if (lane == 0) big[1 + atomicAdd(big, 1u)] = (uint32_t)t;
-    return;
+  const uint64_t t0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + warp) * per;
+  const uint32_t count = lane < per && t0 + lane < n_tiles ? tile_count[t0 + lane] : 0u;
+  uint32_t todo = __ballot_sync(0xffffffffu, count != 0);
+  if (!todo) return;
+  const uint32_t most = __reduce_max_sync(0xffffffffu, count);
+  if (lane == 0 && most > *fullest) atomicMax(fullest, most);  // an old value read only costs an atomic
+  for (; todo; todo &= todo - 1) {
+    const int l = __ffs(todo) - 1;
+    const uint64_t t = t0 + l;
+    const uint32_t n = min(__shfl_sync(0xffffffffu, count, l), cap);
+    if (n > kSmallTile) {
+      if (lane == 0) big[1 + atomicAdd(big, 1u)] = (uint32_t)t;
+      continue;
+    }
+    sort_tile(slots + t * cap, n, t, n_tiles, n_pairs, tile_pair_count, lane);
+    __syncwarp();
   }
-  sort_tile(slots + t * cap, n, t, n_tiles, n_pairs, tile_pair_count, lane);
 }
 
 // The listed tiles, one block of kBigSortThreads each (a tile holds at most kBigSortKeys keys): the
@@ -210,62 +214,65 @@ __global__ void k_emit_hits(const uint64_t* __restrict__ slots, const uint32_t* 
                             const uint64_t* __restrict__ rec_group, uint32_t n_rec, ah_hit* __restrict__ hits,
                             const uint64_t* __restrict__ tile_base = nullptr, uint64_t hit_cap = ~0ull,
                             uint32_t* __restrict__ overflow = nullptr, uint64_t* __restrict__ pair_off = nullptr,
-                            uint32_t n_pairs = 0) {
+                            uint32_t n_pairs = 0, uint32_t per = 1) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (pair_off && blockIdx.x == 0)  // each pair's first hit
     for (uint32_t p = threadIdx.x; p <= n_pairs; p += blockDim.x) pair_off[p] = off[(uint64_t)p * n_tiles];
-  const uint64_t t = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-  if (t >= n_tiles) return;
-  const uint32_t n = min(tile_count[t], cap);
-  if (n == 0) return;
-  const uint64_t* tk = slots + t * cap;
-  const uint64_t tile_pos = tile_base ? tile_base[t] : t * tile_groups * 32ull;
-  // the records the tile's sites fall in, [r_lo, r_hi]: lane 0 finds the one holding the smallest
-  // position, lane 1 the one holding the largest, so a site's record search spans those only
-  uint64_t p_min = ~0ull, p_max = 0;
-  for (uint32_t i = lane; i < n; i += 32) {
-    const uint64_t x = (tk[i] >> 16) & 0xffffffffull;
-    p_min = min(p_min, x);
-    p_max = max(p_max, x);
-  }
+  const uint64_t t0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + warp) * per;
+  const uint32_t count = lane < per && t0 + lane < n_tiles ? tile_count[t0 + lane] : 0u;
+  for (uint32_t todo = __ballot_sync(0xffffffffu, count != 0); todo; todo &= todo - 1) {
+    const int l = __ffs(todo) - 1;
+    const uint64_t t = t0 + l;
+    const uint32_t n = min(__shfl_sync(0xffffffffu, count, l), cap);
+    const uint64_t* tk = slots + t * cap;
+    const uint64_t tile_pos = tile_base ? tile_base[t] : t * tile_groups * 32ull;
+    // the records the tile's sites fall in, [r_lo, r_hi]: lane 0 finds the one holding the smallest
+    // position, lane 1 the one holding the largest, so a site's record search spans those only
+    uint64_t p_min = ~0ull, p_max = 0;
+    for (uint32_t i = lane; i < n; i += 32) {
+      const uint64_t x = (tk[i] >> 16) & 0xffffffffull;
+      p_min = min(p_min, x);
+      p_max = max(p_max, x);
+    }
 #pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    p_min = min(p_min, __shfl_xor_sync(0xffffffffu, p_min, o));
-    p_max = max(p_max, __shfl_xor_sync(0xffffffffu, p_max, o));
-  }
-  uint32_t r = 0;
-  if (lane < 2) {
-    const uint64_t pos = tile_pos + (lane ? p_max : p_min);
-    uint32_t lo = 0, hi = n_rec;
-    while (hi - lo > 1) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (rec_group[mid] * 32ull <= pos) lo = mid; else hi = mid;
+    for (int o = 16; o; o >>= 1) {
+      p_min = min(p_min, __shfl_xor_sync(0xffffffffu, p_min, o));
+      p_max = max(p_max, __shfl_xor_sync(0xffffffffu, p_max, o));
     }
-    r = lo;
-  }
-  const uint32_t r_lo = __shfl_sync(0xffffffffu, r, 0), r_hi = __shfl_sync(0xffffffffu, r, 1);
-  const bool one_pair = (tk[0] >> 48) == (tk[n - 1] >> 48);  // keys are sorted by pair first
-  for (uint32_t i = lane; i < n; i += 32) {
-    const uint64_t key = tk[i];
-    const uint32_t pair = (uint32_t)(key >> 48);
-    const uint32_t first = one_pair ? 0u : lower_bound_u64(tk, n, (uint64_t)pair << 48);
-    const uint64_t o = off[(uint64_t)pair * n_tiles + t] + (i - first);
-    const uint64_t pos = tile_pos + ((key >> 16) & 0xffffffffull);
-    uint32_t lo = r_lo, hi = r_hi + 1;
-    while (hi - lo > 1) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (rec_group[mid] * 32ull <= pos) lo = mid; else hi = mid;
+    uint32_t r = 0;
+    if (lane < 2) {
+      const uint64_t pos = tile_pos + (lane ? p_max : p_min);
+      uint32_t lo = 0, hi = n_rec;
+      while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (rec_group[mid] * 32ull <= pos) lo = mid; else hi = mid;
+      }
+      r = lo;
     }
-    ah_hit h;
-    h.record = lo;
-    h.pos = (uint32_t)(pos - rec_group[lo] * 32ull);
-    h.pattern = (uint16_t)(pair * 4u + ((key >> 8) & 3u));
-    h.mism = (uint8_t)(key & 0xffu);
-    h.flags = 0;
-    if (o < hit_cap)
-      hits[o] = h;
-    else if (overflow)
-      atomicOr(overflow, 2u);
+    const uint32_t r_lo = __shfl_sync(0xffffffffu, r, 0), r_hi = __shfl_sync(0xffffffffu, r, 1);
+    const bool one_pair = (tk[0] >> 48) == (tk[n - 1] >> 48);  // keys are sorted by pair first
+    for (uint32_t i = lane; i < n; i += 32) {
+      const uint64_t key = tk[i];
+      const uint32_t pair = (uint32_t)(key >> 48);
+      const uint32_t first = one_pair ? 0u : lower_bound_u64(tk, n, (uint64_t)pair << 48);
+      const uint64_t o = off[(uint64_t)pair * n_tiles + t] + (i - first);
+      const uint64_t pos = tile_pos + ((key >> 16) & 0xffffffffull);
+      uint32_t lo = r_lo, hi = r_hi + 1;
+      while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (rec_group[mid] * 32ull <= pos) lo = mid; else hi = mid;
+      }
+      ah_hit h;
+      h.record = lo;
+      h.pos = (uint32_t)(pos - rec_group[lo] * 32ull);
+      h.pattern = (uint16_t)(pair * 4u + ((key >> 8) & 3u));
+      h.mism = (uint8_t)(key & 0xffu);
+      h.flags = 0;
+      if (o < hit_cap)
+        hits[o] = h;
+      else if (overflow)
+        atomicOr(overflow, 2u);
+    }
   }
 }
 
@@ -475,17 +482,14 @@ void launch_scan_range(cudaStream_t s, const ScanKernel& k, const ah_batch* b, u
   cudaLaunchKernel((const void*)k.fn, dim3((unsigned)((g1 - g0 + bg - 1) / bg)), dim3((unsigned)k.threads), args, 0, s);
 }
 
-void launch_tile_max(cudaStream_t s, const uint32_t* tile_count, uint64_t n_tiles, uint32_t* out) {
-  k_tile_max<<<std::max<uint64_t>(1, std::min<uint64_t>(1024, (n_tiles + 255) / 256)), 256, 0, s>>>(tile_count, n_tiles,
-                                                                                                     out);
-}
-
 // sort every tile's keys and count them per pair; `big` (n_tiles + 1 words) is needed only when
 // cap > kSmallTile
 int launch_tile_sort(cudaStream_t s, uint64_t* slots, const uint32_t* tile_count, uint32_t cap, uint64_t n_tiles,
-                     uint32_t n_pairs, uint32_t* tpc, uint32_t* big, int sm_count) {
+                     uint32_t n_pairs, uint32_t* tpc, uint32_t* big, int sm_count, uint32_t* fullest) {
   if (cap > kSmallTile) cudaMemsetAsync(big, 0, sizeof(uint32_t), s);
-  k_tile_sort<<<(unsigned)((n_tiles + 7) / 8), 256, 0, s>>>(slots, tile_count, cap, n_tiles, n_pairs, tpc, big);
+  const uint32_t per = tiles_per_warp(n_tiles);
+  k_tile_sort<<<(unsigned)((n_tiles + 8 * per - 1) / (8 * per)), 256, 0, s>>>(slots, tile_count, cap, n_tiles, n_pairs, tpc,
+                                                                              big, per, fullest);
   if (cap <= kSmallTile) return 1;
   const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(n_tiles, 4ull * (uint64_t)std::max(1, sm_count)));
   k_tile_sort_big<<<grid, kBigSortThreads, 0, s>>>(slots, tile_count, cap, n_tiles, n_pairs, tpc, big);
@@ -496,9 +500,10 @@ void launch_emit_hits(cudaStream_t s, const uint64_t* slots, const uint32_t* til
                       uint64_t tile_groups, const uint64_t* off, const ah_batch* b, ah_hit* hits,
                       const uint64_t* tile_base, uint64_t hit_cap, uint32_t* overflow, uint64_t* pair_off,
                       uint32_t n_pairs) {
-  k_emit_hits<<<(unsigned)((n_tiles + 7) / 8), 256, 0, s>>>(slots, tile_count, cap, n_tiles, tile_groups, off,
-                                                            b->rec_group, b->n_records, hits, tile_base, hit_cap, overflow,
-                                                            pair_off, n_pairs);
+  const uint32_t per = tiles_per_warp(n_tiles);
+  k_emit_hits<<<(unsigned)((n_tiles + 8 * per - 1) / (8 * per)), 256, 0, s>>>(
+      slots, tile_count, cap, n_tiles, tile_groups, off, b->rec_group, b->n_records, hits, tile_base, hit_cap, overflow,
+      pair_off, n_pairs, per);
 }
 
 namespace {
@@ -732,8 +737,7 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
     cudaMemsetAsync(d_max, 0, sizeof(uint32_t), ctx->stream);
     cudaMemsetAsync(tpc, 0, n_cells * sizeof(uint32_t), ctx->stream);
     if ((st = launch_scan(ctx, b, p, cfg, per_record, tile_groups, n_tiles, slots, tile_count, cap))) return done(st);
-    launch_tile_max(ctx->stream, tile_count, n_tiles, d_max);
-    launched(ctx, 1 + launch_tile_sort(ctx->stream, slots, tile_count, cap, n_tiles, n_pairs, tpc, big, ctx->sm_count));
+    launched(ctx, launch_tile_sort(ctx->stream, slots, tile_count, cap, n_tiles, n_pairs, tpc, big, ctx->sm_count, d_max));
     if ((st = exclusive_scan_u32(ctx, tpc, off, n_cells))) return done(st);
     k_scan_summary<<<1, 256, 0, ctx->stream>>>(off, n_tiles, n_pairs, d_max, ctx->d_status, h->d_pair_off, ctx->h_read);
     launched(ctx);
@@ -767,8 +771,8 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
   h->n = h->h_pair_off[n_pairs];
   if ((st = dalloc(ctx, &h->d, h->n))) return done(st);
   if (h->n) {
-    k_emit_hits<<<(unsigned)((n_tiles + 7) / 8), 256, 0, ctx->stream>>>(slots, tile_count, cap, n_tiles, tile_groups, off,
-                                                                        b->rec_group, b->n_records, h->d);
+    launch_emit_hits(ctx->stream, slots, tile_count, cap, n_tiles, tile_groups, off, b, h->d, nullptr, ~0ull, nullptr,
+                     nullptr, n_pairs);
     launched(ctx);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return done(fail(ctx, AH_ECUDA, "site emission failed: %s", cudaGetErrorString(e)));
