@@ -1855,11 +1855,14 @@ int launch_tm_hits(cudaStream_t s, const TmRun& R, const ah_primers* p, const ah
   int n_launched = 0;
   if (const size_t smem = thread_kernel_smem(p, R.variants)) {
     cudaMemsetAsync(defer, 0, sizeof(uint32_t), s);
-    // fewer sites: smaller windows, down to one site per thread, until sixteen blocks per SM have work (a thread takes
-    // its share of a window's sites one after another, a chain of some 12 us each).  344,000 slots of reads 75 -> 43 us
-    // (four blocks per SM: 50), 38,000 slots 58 -> 18, 11,000 slots of eight pairs 69 -> 26; below 128 slots nothing more.
+    // fewer sites: smaller windows, down to one site per thread, until four blocks per SM have work (a thread takes its
+    // share of a window's sites one after another, a chain of some 10 us each).  38,000 slots 58 -> 18 us, 11,000 slots
+    // of eight pairs 69 -> 26, 344,000 slots of reads 75 -> 50, 83,000 to 614,000 slots of repeats 82 -> 30 to 124 -> 98
+    // (937,000, windows of 1,024 either way: 147).  Every block also fills its tables, so windows that make
+    // more blocks than the SMs hold at once (eight each) lose: 2.8 million slots of repeats take 372 us in windows of
+    // 1,024, 442 of 512 and 868 of 128.
     int window = kTmSlots;
-    while (window > kTmThreads && cap < 16ull * (uint64_t)std::max(1, sm_count) * (uint64_t)window) window /= 2;
+    while (window > kTmThreads && cap < 4ull * (uint64_t)std::max(1, sm_count) * (uint64_t)window) window /= 2;
     const unsigned grid = (unsigned)std::max<uint64_t>(1, (cap + window - 1) / window);
     const size_t smem_j = 4 * ((size_t)kTmThreadFixedWords + (size_t)tk.weight_words * kTmThreads);
     if (tk.fn && tk.image && smem_j <= kTmSmemCap) {  // the kernel generated for this primer set
