@@ -93,6 +93,11 @@ SCAN_TRAFFIC = {
     # autotuner keeps, registers bounded for 4 blocks per SM)
     (996, 128, 8, 0, 0): ((873_291_008 + 743_168) / 3_487_157_421,
                           "the batched set's first 2,000 genomes (profiles/ah_scan_jit_alu_pipe.md)"),
+    # the interleaved form, which plans choose: the same two cases
+    (71, 64, 32, 0, 0): ((189_601_792 + 191_488) / 756_529_120,
+                         "plain_scale's first 200 genomes (profiles/ah_scan_jit_alu_pipe.md)"),
+    (324, 64, 32, 0, 0): ((873_364_480 + 598_272) / 3_487_157_421,
+                          "the batched set's first 2,000 genomes (profiles/ah_scan_jit_alu_pipe.md)"),
 }
 
 
@@ -106,6 +111,13 @@ SCAN_PIPE = {
     186: {"alu_lane_ops_per_base": 109_810_167 * 32 / 756_529_120, "alu_pipe_busy": 0.966,
           "source": "ncu smsp__inst_executed_pipe_alu.sum x 32 / bases of one launch, plain_scale 200 genomes "
                     "(profiles/ah_scan_jit_alu_pipe.md)"},
+    # the interleaved form on the same cases: 59,262,158 and 1,065,948,134 ALU-pipe warp instructions
+    71: {"alu_lane_ops_per_base": 59_262_158 * 32 / 756_529_120, "alu_pipe_busy": 0.844,
+         "source": "ncu smsp__inst_executed_pipe_alu.sum x 32 / bases of one launch, plain_scale 200 genomes, interleaved "
+                   "form (profiles/ah_scan_jit_alu_pipe.md)"},
+    324: {"alu_lane_ops_per_base": 1_065_948_134 * 32 / 3_487_157_421, "alu_pipe_busy": 0.818,
+          "source": "ncu smsp__inst_executed_pipe_alu.sum x 32 / bases of one launch, batched 2,000 genomes, interleaved "
+                    "form (profiles/ah_scan_jit_alu_pipe.md)"},
     # the batched set (8 pairs = 32 patterns, k = i mod 4): its first 2,000 genomes (3.49 Gbp), the
     # kernel the autotuner keeps: 128 threads x 8 groups, shift mode 0, registers bounded for 4 blocks
     # per SM, phase split drawn for 4,096 windows per vote (996 LOP3/SHF per 32 positions);
