@@ -393,7 +393,7 @@ void launch_tm(cudaStream_t s, const void* run, const ah_hit* hits, uint64_t hit
                uint32_t* defer, int sm_count, const TmKernel& tk,
                bool marked = false, bool sites_only = false);
 // Plans with few sites and amplicons: the pairing (both walks, the scan between them, the marking of the sites whose
-// Tm is wanted) and what follows the Tm stage up to the extraction (threshold, compaction, lengths, their scan) in one
+// Tm is wanted, the deferred list emptied) and what follows the Tm stage up to the extraction (threshold, compaction, lengths, their scan) in one
 // block each.  total: the amplicons found; ebase (may be null): offsets of the kept amplicons' bytes and their total.
 // (A replay with 64 sites takes 53 us this way and 69 over many blocks, with 2,048 sites 96 and 105, with 4,096 110 and
 // 108; a plan that sizes its own buffers at 4,096 holds up to 2,457.)
@@ -401,7 +401,7 @@ constexpr uint64_t kOneBlockItems = 4096;
 constexpr unsigned long long kWantedMark = 0xFFFFFFFFFFFFFFFFull;  // the Tm kernels' kSiteWanted
 void launch_pairs_one(cudaStream_t s, const ah_hit* hits, uint64_t cap, const uint64_t* d_n, const uint64_t* pair_off,
                       const uint8_t* plen, uint32_t min_len, uint32_t max_len, uint32_t mask, ah_amplicon* out,
-                      uint64_t out_cap, uint32_t* overflow, double* hit_tm, uint64_t* total);
+                      uint64_t out_cap, uint32_t* overflow, double* hit_tm, uint32_t* defer, uint64_t* total);
 void launch_finish_one(cudaStream_t s, ah_amplicon* amps, uint64_t cap, const uint64_t* d_n, const double* hit_tm,
                        int filter, double min_tm, ah_amplicon* kept, uint64_t* n_kept, const ah_hit* hits,
                        const uint32_t* rec_len, const uint8_t* plen, int trim, uint32_t fb, uint32_t rb, uint64_t* ebase);

@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kOneThreads) k_pairs_one(
     const ah_hit* __restrict__ hits, uint64_t cap, const uint64_t* __restrict__ d_n, const uint64_t* __restrict__ pair_off,
     const uint8_t* __restrict__ plen, uint32_t min_len, uint32_t max_len, uint32_t mask, ah_amplicon* __restrict__ out,
     uint64_t out_cap, uint32_t* __restrict__ overflow, unsigned long long* __restrict__ hit_tm,
-    uint64_t* __restrict__ total) {
+    uint32_t* __restrict__ defer, uint64_t* __restrict__ total) {
   __shared__ uint32_t sums[kOneThreads / 32];
   const uint64_t n = min(*d_n, cap);
   for (uint64_t i = threadIdx.x; i < cap; i += kOneThreads) hit_tm[i] = 0;
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kOneThreads) k_pairs_one(
                     hit_tm);
     carry += all;
   }
-  if (threadIdx.x == 0) *total = carry;
+  if (threadIdx.x == 0) *total = carry, *defer = 0;
 }
 
 }  // namespace
@@ -158,9 +158,9 @@ void launch_pair_walk(cudaStream_t s, bool emit, const ah_hit* hits, uint64_t ca
 
 void launch_pairs_one(cudaStream_t s, const ah_hit* hits, uint64_t cap, const uint64_t* d_n, const uint64_t* pair_off,
                       const uint8_t* plen, uint32_t min_len, uint32_t max_len, uint32_t mask, ah_amplicon* out,
-                      uint64_t out_cap, uint32_t* overflow, double* hit_tm, uint64_t* total) {
+                      uint64_t out_cap, uint32_t* overflow, double* hit_tm, uint32_t* defer, uint64_t* total) {
   k_pairs_one<<<1, kOneThreads, 0, s>>>(hits, cap, d_n, pair_off, plen, min_len, max_len, mask, out, out_cap, overflow,
-                                        reinterpret_cast<unsigned long long*>(hit_tm), total);
+                                        reinterpret_cast<unsigned long long*>(hit_tm), defer, total);
 }
 
 ah_status pair_amplicons(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const ah_hits* h, uint32_t min_len,

@@ -1850,11 +1850,12 @@ size_t thread_kernel_smem(const ah_primers* p, int variants) {
 // lists them there for k_tm_deferred).  Returns the kernels launched.
 int launch_tm_hits(cudaStream_t s, const TmRun& R, const ah_primers* p, const ah_hit* hits, uint64_t cap,
                     const uint64_t* d_n, const uint2* planes, const uint64_t* rec_group, double* hit_tm,
-                    uint32_t* status, uint32_t* defer, int sm_count, const TmKernel& tk, bool* generated) {
+                    uint32_t* status, uint32_t* defer, int sm_count, const TmKernel& tk, bool* generated,
+                    bool emptied = false) {
   if (generated) *generated = false;
   int n_launched = 0;
   if (const size_t smem = thread_kernel_smem(p, R.variants)) {
-    cudaMemsetAsync(defer, 0, sizeof(uint32_t), s);
+    if (!emptied) cudaMemsetAsync(defer, 0, sizeof(uint32_t), s);
     // fewer sites: smaller windows, down to one site per thread, until four blocks per SM have work (a thread takes its
     // share of a window's sites one after another, a chain of some 10 us each).  38,000 slots 58 -> 18 us, 11,000 slots
     // of eight pairs 69 -> 26, 344,000 slots of reads 75 -> 50, 83,000 to 614,000 slots of repeats 82 -> 30 to 124 -> 98
@@ -2044,7 +2045,7 @@ void launch_tm(cudaStream_t s, const void* run, const ah_hit* hits, uint64_t hit
     cudaMemsetAsync(hit_tm, 0, std::max<uint64_t>(1, hit_cap) * sizeof(double), s);
     k_mark_sites<<<(unsigned)std::max<uint64_t>(1, (amp_cap + 255) / 256), 256, 0, s>>>(amps, amp_cap, hit_tm, d_namps);
   }
-  launch_tm_hits(s, R, p, hits, hit_cap, d_nhits, planes, rec_group, hit_tm, status, defer, sm_count, tk, nullptr);
+  launch_tm_hits(s, R, p, hits, hit_cap, d_nhits, planes, rec_group, hit_tm, status, defer, sm_count, tk, nullptr, marked);
   if (sites_only) return;
   k_tm_amps<<<(unsigned)std::max<uint64_t>(1, (amp_cap + 255) / 256), 256, 0, s>>>(amps, amp_cap, hit_tm, filter,
                                                                                   min_tm, keep, d_namps);
