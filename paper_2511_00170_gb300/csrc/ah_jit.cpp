@@ -984,7 +984,8 @@ std::string interleaved_source(const std::vector<Pattern>& pats, const ScanConfi
   }
   os << body;
   os << "    if (!care) {\n      i0 += " << R << ";\n      continue;\n    }\n";
-  os << "    __syncwarp();\n    const u32 n = qu.n;\n";
+  // (read by every lane before any lane adds to it again: the whole warp goes one way from here)
+  os << "    __syncwarp();\n    const u32 n = qu.n;\n    __syncwarp();\n";
   os << "    if (sel == ~0u && n <= QCAP / 2) {\n      i0 += " << R << ";\n      continue;\n    }\n";
   os << "    const bool again = sel == ~0u && n > QCAP;\n";
   os << "    drain(min(n, (u32)QCAP), again ? i0 : 32u, first, P, qu.w, qu.m);\n    __syncwarp();\n";

@@ -1,0 +1,152 @@
+"""The interleaved scan form on the CPU: the generated kernel's own text, compiled for the host and run a warp at a
+time with every lane as a fiber (warp_emulator.h), finds exactly the windows that a per-position count and clamp check
+finds.  It runs with its lanes in several orders between two warp-wide operations, so that a result that rests on a
+warp staying converged shows.  It also compiles for sm_103a (NVRTC on the host).  No GPU is needed."""
+import os
+import re
+import subprocess
+
+import numpy as np
+import pytest
+
+import synth
+from tests.scan_emulator import CODE, COMP, SETS
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+BUILD = os.path.join(ROOT, "paper_2511_00170_gb300", "_build")
+TESTS = os.path.join(ROOT, "tests")
+
+EIGHT = ["CGATANRNCGCGCCRCATMGTA", "MYGTGCTGYCACAACRCGA", "GTYAGCAAWGCACTCGMAAC", "GGCGMCGCGGGTYACRGTTGA",
+         "CNGRRTATATSARCWGTATC", "CTAACCGGTAAACACTCACGA", "AGCGCTCAGTACAGCTAT", "TGCARTGAATCCTCWGCAGCCT",
+         "GTRTGGGAGTGGTRAGTCGNTTACA", "CAGCAGTTCGGRTGCTCTGG", "CCGGCGTGTAGATCCTGTGATTA",
+         "GGGCGTKTAGTGTSTGTTGTACACT", "AGGGSMGMAAGARARCMCGA", "TTAGCACWGATTTSGAACCAG", "CACKANCRKACCRCCCACA",
+         "SGKGAATAGTTTARWTGTAG"]
+PLAIN = ["AGATACCKWCAACAACTGC", "CTCCTCGTATAWTMTCRACC"]
+
+
+@pytest.fixture(scope="module")
+def dump():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    exe, lib = os.path.join(BUILD, "il_dump"), os.path.join(ROOT, "paper_2511_00170_gb300")
+    sources = [os.path.join(TESTS, "il_dump.cpp"), os.path.join(TESTS, "jit_dump.cpp")]
+    if not os.path.exists(exe) or os.path.getmtime(exe) < max(map(os.path.getmtime, sources + [f"{lib}/libah.so"])):
+        subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", "/usr/local/cuda/include", sources[0], "-o", exe,
+                               "-L", lib, "-lah", f"-Wl,-rpath,{lib}"])
+
+    def run(what, k, clamp, primers, windows=1024):
+        return subprocess.run([exe, what, f"windows={windows}", str(k), str(clamp)] + primers, text=True,
+                              capture_output=True, check=what != "compile").stdout
+
+    return run
+
+
+def host_source(src):
+    """The generated text as C++ for warp_emulator.h."""
+    src = re.sub(r'asm\("lop3\.b32 %0, %1, %2, %3, (0x[0-9a-f]+);" : "=r"\((\w+)\) : "r"\(([\w.]+)\), "r"\(([\w.]+)\), '
+                 r'"r"\(([\w.]+)\)\);', r"\2 = lop3(\3, \4, \5, \1);", src)
+    src = re.sub(r'asm volatile\("prefetch[^;]*;"[^;]*;', ";", src)
+    assert 'asm("' not in src
+    with open(os.path.join(TESTS, "il_run.cpp")) as f:
+        return '#include "warp_emulator.h"\n' + src + f.read()
+
+
+def build(tmp, src):
+    cpp, exe = os.path.join(tmp, "kernel.cpp"), os.path.join(tmp, "kernel")
+    with open(cpp, "w") as f:
+        f.write(host_source(src))
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-w", "-I", TESTS, cpp, "-o", exe])
+    return exe
+
+
+def planes_of(text):
+    """Text (ACGT, anything else invalid) to plane and invalid words of whole groups, and 64 groups after them."""
+    b = np.frombuffer(text.encode(), dtype=np.uint8)
+    n = (len(b) + 31) // 32
+    code, bad = np.zeros(n * 32, np.uint8), np.ones(n * 32, bool)
+    for c, v in CODE.items():
+        m = np.flatnonzero(b == ord(c))
+        code[m], bad[m] = v, False
+    word = lambda bits: np.packbits(bits.astype(np.uint8), bitorder="little").view(np.uint32)
+    planes = np.zeros((n + 64, 2), np.uint32)
+    invalid = np.full(n + 64, 0xFFFFFFFF, np.uint32)
+    planes[:n, 0], planes[:n, 1], invalid[:n] = word(code & 1), word(code >> 1), word(bad)
+    return n, planes, invalid, code, bad
+
+
+def run(exe, tmp, text, cap=1 << 17, order=0, first=0, count=None):
+    """(returncode, status, tile counts, sorted sites (tile, key))"""
+    n, planes, invalid, _, _ = planes_of(text)
+    count = n - first if count is None else count
+    a, b = os.path.join(tmp, "in"), os.path.join(tmp, "out")
+    with open(a, "wb") as f:
+        f.write(np.array([n, first, count, cap], np.uint32).tobytes() + planes.tobytes() + invalid.tobytes())
+    r = subprocess.run([exe, a, b, str(order)], capture_output=True, text=True, timeout=300)
+    if r.returncode:
+        return r.returncode, r.stderr, None, None
+    raw = np.fromfile(b, np.uint8)
+    tiles = (n + 1023) // 1024
+    status = int(raw[:4].view(np.uint32)[0])
+    counts = raw[4:4 + 4 * tiles].view(np.uint32)
+    slots = raw[4 + 4 * tiles:].view(np.uint64).reshape(tiles, cap)
+    sites = sorted((t, int(s)) for t in range(tiles) for s in slots[t, :min(cap, counts[t])])
+    return 0, status, counts, sites
+
+
+def expected(text, primers, k, clamp):
+    n, _, _, code, bad = planes_of(text)
+    code, bad = np.pad(code, (0, 64)), np.pad(bad, (0, 64), constant_values=True)
+    out, x = [], np.arange(n * 32)
+    q = 0
+    for p in primers:
+        p, kk = (p.split(":")[0], int(p.split(":")[1])) if ":" in p else (p, k)
+        rc = "".join(COMP[c] for c in reversed(p))
+        for pat, cl in ((p, range(len(p) - clamp, len(p))), (rc, range(0, clamp))):
+            mism, ok = np.zeros(n * 32, int), np.ones(n * 32, bool)
+            for j, ch in enumerate(pat):
+                match = np.isin(code[x + j], [CODE[c] for c in SETS[ch]])
+                mism += ~match
+                ok &= ~bad[x + j]
+                if j in cl:
+                    ok &= match
+            for pos in np.flatnonzero(ok & (mism <= kk)):
+                t = int(pos) // 32768
+                out.append((t, (q // 4) << 48 | (int(pos) - t * 32768) << 16 | (q % 4) << 8 | int(mism[pos])))
+            q += 1
+    return sorted(out)
+
+
+def _random(n, seed):
+    return "".join(np.array(list("ACGT"))[np.random.default_rng(seed).integers(0, 4, n)])
+
+
+def _repeats(n, seed, primers, share):
+    """Random bases with tandem repeats of a primer's concrete bases in `share` of them, and some Ns."""
+    rng = np.random.default_rng(seed)
+    out = list(_random(n, seed))
+    while share > 0:
+        p = primers[int(rng.integers(len(primers)))].split(":")[0]
+        if rng.random() < 0.5:
+            p = "".join(COMP[c] for c in reversed(p))
+        unit = "".join(SETS[c][0] for c in p)
+        m = int(min(n, rng.integers(200, 3000)))
+        at = int(rng.integers(0, n - m + 1))
+        out[at:at + m] = (unit * (m // len(unit) + 1))[:m]
+        share -= m / n
+    for at in rng.integers(0, n, 5):
+        out[at] = "N"
+    return "".join(out)
+
+
+@pytest.mark.parametrize("order", [0, 1, 2, 3])
+@pytest.mark.parametrize("k,primers", [(3, PLAIN), (2, EIGHT[:8]), (0, ["ACGTACGT"])])
+def test_queue_overflow_with_lanes_in_any_order(dump, tmp_path, k, primers, order):
+    """Tiles whose surviving windows overflow the warp's queue many times over: the careful mode, in which the queue's
+    length is read after every iteration and decides for the whole warp how it goes on."""
+    exe = build(str(tmp_path), dump("source", k, 3, primers))
+    text = _repeats(50_000, 7 + k, primers, 0.4)
+    rc, status, counts, sites = run(exe, str(tmp_path), text, order=order)
+    assert rc == 0, status
+    want = expected(text, primers, k, 3)
+    assert len(want) > 4 * 96 and sites == want  # the queue holds 96, the text is two tiles
