@@ -335,7 +335,7 @@ ah_status ah_scan_primers_per_record(ah_ctx* ctx, const ah_batch* b, const ah_pr
 
 ah_status ah_hits_count(const ah_hits* h, uint64_t* n);
 /* Device view: hits in device memory (ah_hit[n]) and, per pair, the range of its hits
- * (uint64[n_pairs+1], device). */
+ * (uint64[n_pairs+1], device).  Waits until they are written: any stream may read them then. */
 ah_status ah_hits_device(const ah_hits* h, const ah_hit** d_hits, const uint64_t** d_pair_offsets);
 /* Copy min(n, cap) hits to host memory; synchronises. */
 ah_status ah_hits_copy(const ah_hits* h, ah_hit* host_out, uint64_t cap);

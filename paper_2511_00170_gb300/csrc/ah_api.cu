@@ -1173,6 +1173,13 @@ ah_status ah_hits_count(const ah_hits* h, uint64_t* n) {
 
 ah_status ah_hits_device(const ah_hits* h, const ah_hit** d_hits, const uint64_t** d_pair_offsets) {
   if (!h) return AH_EINVAL;
+  if (h->written) {  // the caller may read the sites on a stream of its own, also while it captures one
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaEventSynchronize(h->written);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return fail(h->ctx, AH_ECUDA, "ah_hits_device: %s", cudaGetErrorString(e));
+  }
   if (d_hits) *d_hits = h->d;
   if (d_pair_offsets) *d_pair_offsets = h->d_pair_off;
   return AH_OK;
@@ -1188,6 +1195,7 @@ void ah_hits_free(ah_hits* h) {
   if (!h) return;
   dfree(h->ctx, h->d);
   dfree(h->ctx, h->d_pair_off);
+  if (h->written) cudaEventDestroy(h->written);
   delete h;
 }
 

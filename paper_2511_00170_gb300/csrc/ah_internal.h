@@ -206,6 +206,7 @@ struct ah_hits {
   ah_hit* d = nullptr;
   uint64_t* d_pair_off = nullptr;      // n_pairs + 1
   std::vector<uint64_t> h_pair_off;
+  cudaEvent_t written = nullptr;       // the emission's end where the scan returned before it (ah_hits_device waits)
 };
 
 struct ah_amplicons {

@@ -774,7 +774,10 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
     launch_emit_hits(ctx->stream, slots, tile_count, cap, n_tiles, tile_groups, off, b, h->d, nullptr, ~0ull, nullptr,
                      nullptr, n_pairs);
     launched(ctx);
-    const cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    // the context's own calls are ordered after the emission; a reader on another stream waits for it
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->written, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(h->written, ctx->stream);
     if (e != cudaSuccess) return done(fail(ctx, AH_ECUDA, "site emission failed: %s", cudaGetErrorString(e)));
   }
   return done(AH_OK);
