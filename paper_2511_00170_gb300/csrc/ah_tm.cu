@@ -913,8 +913,7 @@ __device__ double group_site_tm(TmGroupSh& sh, int32_t* w, int L, int k, int cla
     fixed_gc |= __shfl_xor_sync(gmask, fixed_gc, o, G);
   }
   if (empty) return nan;
-  const int m0 = __popc(fixed_mm);
-  if (K >= 0 && m0 > K) return nan;
+  if (K >= 0 && __popc(fixed_mm) > K) return nan;
   __syncwarp(gmask);  // ch is read by the whole group
   const bool flat = R.saltcorr >= 6 && L >= 3;  // enumerated by the group, unless too many combinations
   uint32_t combos = 1;
@@ -936,6 +935,7 @@ __device__ double group_site_tm(TmGroupSh& sh, int32_t* w, int L, int k, int cla
   }
   if (!dmask) dmask = 1;  // a concrete primer: a chain of one node with a single choice
   const int D = __popc(dmask);
+  const int m0 = __popc(fixed_mm & ~dmask);  // the chain's nodes count their own mismatches
   for (int t = r; t < D; t += G) {  // the t-th set bit of dmask
     uint32_t x = dmask;
     for (int q = 0; q < t; ++q) x &= x - 1;
@@ -991,7 +991,7 @@ __device__ double group_site_tm(TmGroupSh& sh, int32_t* w, int L, int k, int cla
     }
   }
   __syncwarp(gmask);
-  if (flat) return group_enum_max<G>(sh, w, D, combos, K, __popc(fixed_mm & ~dmask), __popc(fixed_gc & ~dmask), L, R, r, gmask);
+  if (flat) return group_enum_max<G>(sh, w, D, combos, K, m0, __popc(fixed_gc & ~dmask), L, R, r, gmask);
   // a bound on every variant's dS: each step's largest (tenths)
   int bound = 0;
   for (int t = r; t + 1 < D; t += G) {
