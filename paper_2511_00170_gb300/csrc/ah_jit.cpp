@@ -761,10 +761,22 @@ static __device__ __forceinline__ void transpose32(u32 (&a)[32]) {
   SWAP_BITS(1, 0x55555555u)
 }
 
+// The mismatches of pattern q's window at position i of group g, a bit per pattern position, from the
+// bases and per-position set masks.
+static __device__ __forceinline__ u32 mismatches(int q, u32 i, u64 g, const ScanParams& P) {
+  const uint2 x = __ldg(P.planes + g), y = __ldg(P.planes + g + 1);
+  const u64 lo64 = (u64)x.x | ((u64)y.x << 32), hi64 = (u64)x.y | ((u64)y.y << 32);
+  const u32 wl = (u32)(lo64 >> i), wh = (u32)(hi64 >> i);  // base j of the window at bit j
+  const u32 match = (~wl & ~wh & MSET[q][0]) | (wl & ~wh & MSET[q][1]) | (~wl & wh & MSET[q][2]) |
+                    (wl & wh & MSET[q][3]);
+  return ~match & (PLEN[q] == 32 ? 0xffffffffu : ((1u << PLEN[q]) - 1u));
+}
+
 // Windows of pattern q at position i of the groups of lane ln (bits of h): decided exactly from the
 // bases against per-position set masks, the mismatches counted by popcount, then the invalid-base
 // test (every record ends in an invalid padding base, so it covers record bounds too), and the
-// sites appended to their tile's slots.  The whole warp takes part, one window per lane and round.
+// sites appended to their tile's slots; a mismatch in the clamp, which every filter tests, sets the
+// status.  The whole warp takes part, one window per lane and round.
 static __device__ __forceinline__ void check_words(u32 h, int q, u32 i, u32 ln, u64 first, const ScanParams& P) {
   const u32 lane = threadIdx.x & 31u;
   while (__any_sync(0xffffffffu, h != 0)) {
@@ -776,24 +788,19 @@ static __device__ __forceinline__ void check_words(u32 h, int q, u32 i, u32 ln, 
       const u64 gl = first + ln + 32u * b;
       if (gl < P.n_groups) {
         const u64 g = P.group_begin + gl;
-        const uint2 x = __ldg(P.planes + g), y = __ldg(P.planes + g + 1);
-        const u64 lo64 = (u64)x.x | ((u64)y.x << 32), hi64 = (u64)x.y | ((u64)y.y << 32);
-        const int L = PLEN[q];
-        const u32 wm = L == 32 ? 0xffffffffu : ((1u << L) - 1u);
-        const u32 wl = (u32)(lo64 >> i), wh = (u32)(hi64 >> i);  // base j of the window at bit j
-        const u32 match = (~wl & ~wh & MSET[q][0]) | (wl & ~wh & MSET[q][1]) | (~wl & wh & MSET[q][2]) |
-                          (wl & wh & MSET[q][3]);
-        const u32 mis = ~match & wm;
+        const u32 mis = mismatches(q, i, g, P);
         const int mism = __popc(mis);
         if (!(mis & PCLAMP[q]) && mism <= PK[q]) {
           const u64 inv64 = (u64)P.invalid[g] | ((u64)P.invalid[g + 1] << 32);
-          if (!((u32)(inv64 >> i) & wm)) {
+          if (!((u32)(inv64 >> i) & (PLEN[q] == 32 ? 0xffffffffu : ((1u << PLEN[q]) - 1u)))) {
             const u64 pos = g * 32ull + (u64)i;
             tile = g / P.tile_groups;
             key = ((u64)PPAIR[q] << 48) | ((pos - tile * P.tile_groups * 32ull) << 16) | ((u64)PORIENT[q] << 8) |
                   (u64)mism;
             ok = true;
           }
+        } else if (mis & PCLAMP[q]) {
+          atomicOr(P.status, 1u);
         }
       }
     }
@@ -806,6 +813,28 @@ static __device__ __forceinline__ void check_words(u32 h, int q, u32 i, u32 ln, 
       base = __shfl_sync(peers, base, leader);
       const u32 idx = base + __popc(peers & ((1u << lane) - 1u));
       if (idx < P.slot_cap) P.slots[tile * (u64)P.slot_cap + idx] = key;
+    }
+  }
+}
+
+// The self-check of the queue's first n entries: every window in them must be one that its filter lets
+// through by design, by the mismatches outside the clamp at the positions that the filter counts, or by its
+// triples with two of three mismatching; a disagreement sets the status.
+static __device__ __noinline__ void verify(u32 n, u64 first, const ScanParams& P, const uint4* qw, const u32* qm) {
+  for (u32 e = threadIdx.x & 31u; e < n; e += 32) {
+    const u32 m = qm[e], i = (m >> 16) & 31u;
+    const uint4 c = qw[e];
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+      const int q = (int)(m & 0xffffu) + t;
+      for (u32 h = t == 0 ? c.x : t == 1 ? c.y : t == 2 ? c.z : c.w; h; h &= h - 1) {
+        const u64 gl = first + (m >> 24) + 32u * (__ffs(h) - 1);
+        if (gl >= P.n_groups) break;
+        const u32 mis = mismatches(q, i, P.group_begin + gl, P);
+        int triples = 0;
+        for (int k = 0; k < MAX_TRIPLES; ++k) triples += __popc(mis & FTRIPLE[q][k]) >= 2;
+        if ((mis & PCLAMP[q]) || __popc(mis & FCOUNTED[q]) > PK[q] || triples >= (PK[q] + 2) / 2) atomicOr(P.status, 1u);
+      }
     }
   }
 }
@@ -826,6 +855,10 @@ static __device__ __noinline__ void drain(u32 n, u32 i_end, u64 first, const Sca
       check_words(h, (int)(m & 0xffffu) + t, (m >> 16) & 31u, m >> 24, first, P);
     }
   }
+  // One block in 128 of a launch checks itself, from the first on: 0.3 % of a replay with one pair, 0.5 %
+  // with eight (one in 16 1.1 and 3.3 %, every window checked where it is decided 3 %: most windows that
+  // come here are refused).
+  if ((blockIdx.x & 127u) == 0u) verify(n, first, P, qw, qm);
 }
 
 // A warp's queue of surviving words: an entry holds a lane's words of a block of four patterns at one
@@ -864,10 +897,30 @@ std::string interleaved_source(const std::vector<Pattern>& pats, const ScanConfi
   os << "// generated scan kernel, interleaved form: " << Q << " patterns\n";
   os << "#define NT " << 32 * kIlWarps << "\n#define QCAP " << kIlQueue << "\n";
   emit_pattern_tables(os, pats);
-  os << kParams << kIlPrelude;
-  // the loop body: R positions of every pattern
   std::vector<IlFilter> filt;
   for (const Pattern& P : pats) filt.push_back(il_filter(P, std::max(1, cfg.vote_windows)));
+  // what each filter tests, for the check: the positions it counts, or its triples
+  int triples = 1;
+  for (const IlFilter& F : filt) triples = std::max(triples, F.triples);
+  os << "#define MAX_TRIPLES " << triples << "\nstatic __device__ const unsigned int FCOUNTED[" << Q << "] = {";
+  for (const IlFilter& F : filt) {
+    uint32_t m = 0;
+    for (int i = 0; i < (F.triples ? 0 : F.n); ++i) m |= 1u << F.counted[i].j;
+    os << m << "u,";
+  }
+  os << "};\nstatic __device__ const unsigned int FTRIPLE[" << Q << "][MAX_TRIPLES] = {";
+  for (const IlFilter& F : filt) {
+    os << "{";
+    for (int t = 0; t < triples; ++t) {
+      uint32_t m = 0;
+      for (int i = 3 * t; i < 3 * t + 3 && t < F.triples; ++i) m |= 1u << F.counted[i].j;
+      os << m << "u,";
+    }
+    os << "},";
+  }
+  os << "};\n";
+  os << kParams << kIlPrelude;
+  // the loop body: R positions of every pattern
   Emitter E;
   std::map<std::pair<int, int>, Val> cache;
   for (int s = 0; s < R; ++s) {

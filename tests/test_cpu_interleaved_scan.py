@@ -150,3 +150,19 @@ def test_queue_overflow_with_lanes_in_any_order(dump, tmp_path, k, primers, orde
     assert rc == 0, status
     want = expected(text, primers, k, 3)
     assert len(want) > 4 * 96 and sites == want  # the queue holds 96, the text is two tiles
+
+
+@pytest.mark.parametrize("clamp", [0, 2])
+@pytest.mark.parametrize("k,primers", [(3, PLAIN), (0, ["ACGTACGT", "NNACGTAC"]), (1, EIGHT[:4]), (5, EIGHT[4:8])])
+def test_self_check(dump, tmp_path, k, primers, clamp):
+    """Windows that a filter lets through by design set no status; with the circuit's verdict altered in one place of
+    the text (one more position let through for every window) the check reports it, and the sites are still right."""
+    src = dump("source", k, clamp, primers)
+    text = _random(33_000, k) + "N" * 7 + _random(500, k + 1)
+    want = expected(text, primers, k, clamp)
+    rc, status, _, sites = run(build(str(tmp_path), src), str(tmp_path), text)
+    assert (rc, status) == (0, 0) and sites == want
+    m = re.search(r"const u32 f1_1 = (\S+);", src)
+    rc, status, _, sites = run(build(str(tmp_path), src.replace(m.group(0), f"const u32 f1_1 = {m.group(1)} & ~2u;")),
+                               str(tmp_path), text)
+    assert (rc, status) == (0, 1) and sites == want
