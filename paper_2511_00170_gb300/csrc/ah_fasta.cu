@@ -614,9 +614,10 @@ ah_status fasta_pack(ah_ctx* ctx, const char* text, uint64_t n_bytes, const uint
                      ah_batch** batch_out, ah_fasta** names_out, const FastaChunkHook* hook = nullptr) {
   cudaSetDevice(ctx->device);
   cudaPointerAttributes pa;
-  const bool on_device = cudaPointerGetAttributes(&pa, text) == cudaSuccess &&
-                         (pa.type == cudaMemoryTypeDevice || pa.type == cudaMemoryTypeManaged);
+  const bool known = cudaPointerGetAttributes(&pa, text) == cudaSuccess;
   cudaGetLastError();
+  const bool on_device = known && (pa.type == cudaMemoryTypeDevice || pa.type == cudaMemoryTypeManaged);
+  const bool page_locked = known && pa.type == cudaMemoryTypeHost;
   ah_status st = AH_OK;
   const uint8_t* t = (const uint8_t*)text;
   uint8_t* staged = nullptr;
@@ -692,26 +693,44 @@ ah_status fasta_pack(ah_ctx* ctx, const char* text, uint64_t n_bytes, const uint
       cudaStreamWaitEvent(cs, ready, 0);
       t = staged;
     }
-    // Copies run ahead of the passes by as many chunks as the call has enqueued: from page-locked memory
-    // all of them at once; from pageable memory a copy returns once it is staged, and the chunk's passes
-    // are enqueued before the next.
-    for (uint64_t t0 = 0, nt; t0 < n_tiles && !st; t0 += nt) {
-      nt = on_device ? n_tiles : next_tiles(n_tiles - t0, hook ? kLeastHookChunk : kLeastChunk);
-      const uint64_t b0 = t0 * kFaTile, nb = std::min(n_bytes, b0 + nt * kFaTile) - b0;
-      if (!on_device) {
+    // Copies run ahead of the passes by as many chunks as the call has enqueued.  Nothing is waited for without a
+    // hook.  With one each chunk's totals are: from page-locked memory all copies are enqueued before, so that the link
+    // never waits for a pass or a hook; from pageable memory, where a copy returns once it is staged, the next
+    // chunk's.  (7.6 GB of FASTA into a plan 36.6 ms; 42.3 with a chunk's copy enqueued after the hook of the one
+    // before.)
+    std::vector<uint64_t> chunk{0};  // first tiles, and the end
+    while (chunk.back() < n_tiles)
+      chunk.push_back(on_device ? n_tiles
+                                : chunk.back() + next_tiles(n_tiles - chunk.back(), hook ? kLeastHookChunk : kLeastChunk));
+    const size_t n_chunks = chunk.size() - 1;
+    std::vector<cudaEvent_t> arrived;
+    auto copy_upto = [&](size_t n) -> ah_status {
+      for (size_t c = arrived.size(); !on_device && c < std::min(n, n_chunks); ++c) {
+        const uint64_t b0 = chunk[c] * kFaTile, b1 = std::min(n_bytes, chunk[c + 1] * kFaTile);
         cudaEvent_t e = nullptr;
-        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess ||
-            cudaMemcpyAsync(staged + b0, text + b0, nb, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
-            cudaEventRecord(e, cs) != cudaSuccess || cudaStreamWaitEvent(ctx->stream, e, 0) != cudaSuccess)
-          st = fail(ctx, AH_ECUDA, "ah_fasta_pack: copy");
-        if (e) landed.push_back(e);
-        if (st) break;
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess)
+          return fail(ctx, AH_ECUDA, "ah_fasta_pack: copy");
+        landed.push_back(e), arrived.push_back(e);
+        if (cudaMemcpyAsync(staged + b0, text + b0, b1 - b0, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
+            cudaEventRecord(e, cs) != cudaSuccess)
+          return fail(ctx, AH_ECUDA, "ah_fasta_pack: copy");
+      }
+      return AH_OK;
+    };
+    for (size_t c = 0; c < n_chunks; ++c) {
+      const uint64_t t0 = chunk[c], nt = chunk[c + 1] - t0;
+      const uint64_t b0 = t0 * kFaTile, nb = std::min(n_bytes, b0 + nt * kFaTile) - b0;
+      if ((st = copy_upto(hook && page_locked ? n_chunks : c + 1))) break;
+      if (!on_device && cudaStreamWaitEvent(ctx->stream, arrived[c], 0) != cudaSuccess) {
+        st = fail(ctx, AH_ECUDA, "ah_fasta_pack: copy");
+        break;
       }
       k_fa_tiles<<<(unsigned)nt, kFaThreads, 0, ctx->stream>>>(t + b0, nb, info + t0);
       k_fa_chain<<<1, kFaThreads, 0, ctx->stream>>>(info + t0, nt, state, tile_entry + t0, seq_base + t0, hdr_base + t0,
                                                     ctx->h_read);
       launched(ctx, 2);
       if (hook) {  // the chunk's totals before its bases are handed on
+        if ((st = copy_upto(c + 2))) break;
         if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) st = fail(ctx, AH_ECUDA, "ah_fasta_pack: parsing failed");
         if (st || (st = grow(ctx->h_read[1]))) break;
         total_seq = ctx->h_read[0], total_hdr = ctx->h_read[1];
