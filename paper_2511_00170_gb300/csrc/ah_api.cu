@@ -12,8 +12,8 @@ using namespace ah;
 // ------------------------------------------------------------------------------------------
 // packing kernels
 //
-// One CTA per item (a piece of one record, at most 2^20 bases), or a warp for short ones; each warp turns
-// 32 groups (1,024 bases) into plane words at a time from 16-byte loads.  The source may be device
+// Windows of consecutive groups to warps, or to eight lanes where records are short; 32 lanes turn 32
+// groups (1,024 bases) into plane words at a time from 16-byte loads.  The source may be device
 // memory or page-locked host memory, which the kernel then reads over the host link.
 namespace {
 
@@ -114,7 +114,7 @@ __device__ __forceinline__ void pack_piece(uintptr_t start, uint64_t n_valid, ui
   }
 }
 
-// A block per item, its warps splitting the item's blocks evenly: the pieces of a staged host chunk.
+// Few items: a block each, its warps splitting the item's blocks evenly.
 __global__ void __launch_bounds__(kPackThreads) k_pack_items(const uint8_t* __restrict__ src,
                                                              const PackItem* __restrict__ items,
                                                              uint2* __restrict__ planes, uint32_t* __restrict__ invalid) {
@@ -127,42 +127,65 @@ __global__ void __launch_bounds__(kPackThreads) k_pack_items(const uint8_t* __re
                  planes + it.dst_group, invalid + it.dst_group);
 }
 
-// Whole records lying end to end (record r's bases at src + rank[r], rec_len[r] of them): every LANES lanes
-// take `window` consecutive groups of the batch, whatever records they belong to, so long records are
-// shared out and short ones gathered, with no list of pieces to build.  Eight lanes where records are
-// short (a 251-base read is 8 groups), so that a warp converts four at a time.
+// What the packing kernel packs: a list of consecutive pieces of the batch's groups, piece r being groups
+// [first, end) whose `len` bases lie at src.
+struct Piece {
+  uint64_t first, end;
+  uintptr_t src;
+  uint64_t len;
+};
+// whole records lying end to end (record r's bases at src + rank[r], rec_len[r] of them)
+struct RecordPieces {
+  const uint8_t* src;
+  const uint64_t *rank, *rec_group;
+  const uint32_t* rec_len;
+  uint64_t n_groups;
+  __device__ uint64_t first(uint32_t r) const { return __ldg(rec_group + r); }
+  __device__ Piece get(uint32_t r, uint32_t n) const {
+    return {first(r), r + 1 < n ? first(r + 1) : n_groups, (uintptr_t)src + __ldg(rank + r), __ldg(rec_len + r)};
+  }
+};
+// pieces of records anywhere (src may be null: offsets are then addresses): a staged host chunk's
+struct ItemPieces {
+  const uint8_t* src;
+  const PackItem* items;
+  __device__ uint64_t first(uint32_t r) const { return __ldg(&items[r].dst_group); }
+  __device__ Piece get(uint32_t r, uint32_t) const {
+    return {first(r), first(r) + __ldg(&items[r].n_groups), (uintptr_t)src + __ldg(&items[r].src_off),
+            __ldg(&items[r].n_valid)};
+  }
+};
+
+// Groups [g_begin, g_end), pieces in their order: every LANES lanes take `window` consecutive groups,
+// whatever pieces they belong to, so long records are shared out and short ones gathered.  Eight lanes
+// where pieces are short (a 251-base read is 8 groups), so that a warp converts four at a time.
 //
-// Bound: HBM, 1.375 bytes per base.  20,011 contigs (1.20 Gbp, 1.65 GB moved): 318 us a call, 5.2 TB/s,
-// 77 % of a copy's rate; 1,200 us with a list of pieces built and uploaded by the host, each letter
-// compared exactly and half the lanes storing.
-template <int LANES>
-__global__ void __launch_bounds__(kPackThreads) k_pack_records(const uint8_t* __restrict__ src,
-                                                               const uint64_t* __restrict__ rank,
-                                                               const uint64_t* __restrict__ rec_group,
-                                                               const uint32_t* __restrict__ rec_len, uint32_t n_rec,
-                                                               uint64_t n_groups, uint32_t window,
-                                                               uint2* __restrict__ planes,
-                                                               uint32_t* __restrict__ invalid) {
+// Bound: HBM, 1.375 bytes per base.  20,011 contigs (1.20 Gbp, 1.65 GB moved): 300 us, 5.5 TB/s, 81 % of a
+// copy's rate.
+template <int LANES, class Pieces>
+__global__ void __launch_bounds__(kPackThreads, 5) k_pack(const Pieces pieces, uint32_t n, uint64_t g_begin, uint64_t g_end,
+                                                       uint32_t window, uint2* __restrict__ planes,
+                                                       uint32_t* __restrict__ invalid) {
   const uint32_t l = threadIdx.x & (LANES - 1);
   const uint32_t mask = LANES == 32 ? 0xffffffffu : ((1u << (LANES & 31)) - 1u) << (threadIdx.x & 31u & ~(LANES - 1u));
-  const uint64_t g0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES * window;
-  if (g0 >= n_groups) return;
-  const uint64_t g1 = min(n_groups, g0 + window);
-  uint32_t lo = 0, hi = n_rec;  // the record that holds group g0
+  const uint64_t g0 = g_begin + ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES * window;
+  if (g0 >= g_end) return;
+  const uint64_t g1 = min(g_end, g0 + window);
+  uint32_t lo = 0, hi = n;  // the piece that holds group g0: every lane probes one place
   while (hi - lo > 1) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (rec_group[mid] <= g0) lo = mid; else hi = mid;
+    const uint32_t step = (hi - lo - 1) / (LANES + 1) + 1;
+    const uint64_t probe = lo + (uint64_t)step * (l + 1);
+    lo += step * __popc(__ballot_sync(mask, probe < hi && pieces.first((uint32_t)probe) <= g0) & mask);
+    hi = (uint32_t)min((uint64_t)hi, (uint64_t)lo + step);
   }
-  for (uint32_t r = lo; r < n_rec; ++r) {
-    const uint64_t first = rec_group[r];
-    if (first >= g1) break;
-    const uint64_t end = r + 1 < n_rec ? rec_group[r + 1] : n_groups;
-    const uint64_t a = max(first, g0), b = min(end, g1);
-    const uint64_t off = (a - first) * kGroupBases, len = rec_len[r];
-    const uint64_t n_valid = off < len ? min(len - off, (b - a) * kGroupBases) : 0;
-    const uint32_t n = (uint32_t)(b - a);
-    pack_piece<LANES>((uintptr_t)src + rank[r] + off, n_valid, n, 0, (n + LANES - 1) / LANES, l, mask, planes + a,
-                      invalid + a);
+  for (uint32_t r = lo; r < n && pieces.first(r) < g1; ++r) {
+    const Piece p = pieces.get(r, n);
+    const uint64_t a = max(p.first, g0), b = min(p.end, g1);
+    if (a >= b) continue;
+    const uint64_t off = (a - p.first) * kGroupBases;
+    const uint64_t n_valid = off < p.len ? min(p.len - off, (b - a) * kGroupBases) : 0;
+    const uint32_t groups = (uint32_t)(b - a);
+    pack_piece<LANES>(p.src + off, n_valid, groups, 0, (groups + LANES - 1) / LANES, l, mask, planes + a, invalid + a);
   }
 }
 
@@ -266,17 +289,16 @@ ah_status layout_batch(ah_ctx* ctx, uint32_t n_rec, const uint64_t* lens, const 
   return AH_OK;
 }
 
+constexpr uint64_t kPieceBases = 1ull << 18;  // bases per item at most (a multiple of 32)
+
 // items for record r's bases [from, to) placed at source offset src_off; the last piece of a
 // record also writes the record's padding groups
 void add_items(std::vector<PackItem>& items, const ah_batch* b, uint32_t r, uint64_t from, uint64_t to,
                uint64_t src_off) {
-  // bases per item (a multiple of 32): a staged chunk of 256 Mi bases is then 1,024 blocks of the
-  // packing kernel, enough to fill the GPU while the next chunk crosses the link
-  const uint64_t piece = 1ull << 18;
   const uint64_t len = b->h_rec_len[r];
   const uint64_t rec_groups = record_groups(len);
-  for (uint64_t a = from; a < to || (a == from && to == from && from == 0 && len == 0); a += piece) {
-    uint64_t e = std::min(to, a + piece);
+  for (uint64_t a = from; a < to || (a == from && to == from && from == 0 && len == 0); a += kPieceBases) {
+    uint64_t e = std::min(to, a + kPieceBases);
     PackItem it;
     it.src_off = src_off + (a - from);
     it.dst_group = b->h_rec_group[r] + a / 32;
@@ -288,32 +310,46 @@ void add_items(std::vector<PackItem>& items, const ah_batch* b, uint32_t r, uint
   }
 }
 
-void launch_pack(cudaStream_t s, const uint8_t* d_src, const PackItem* d_items, size_t n, ah_batch* b, ah_ctx* ctx) {
-  for (size_t i = 0; i < n; i += 0x7fffffff) {
-    const unsigned m = (unsigned)std::min<size_t>(0x7fffffff, n - i);
-    k_pack_items<<<m, kPackThreads, 0, s>>>(d_src, d_items + i, b->planes, b->invalid);
+// groups [g_begin, g_end) from n pieces (see k_pack)
+template <class Pieces>
+void launch_pieces(ah_ctx* ctx, const Pieces& pieces, uint32_t n, uint64_t g_begin, uint64_t g_end, ah_batch* b) {
+  if (g_begin >= g_end) return;
+  // 8 lanes below 16 groups a piece, else 32.  Groups per window, measured: 200,000 reads of 251 bases
+  // with 64 / 32 / 16 / 8 groups 47 / 44 / 48 / 67 us; 20,011 contigs (1.20 Gbp) with 256 / 512 / 1,024 /
+  // 2,048 groups 365 / 329 / 318 / 323 us a call.  Fewer where that leaves SMs without work.
+  const uint64_t groups = g_end - g_begin;
+  const bool narrow = groups < 16ull * n;
+  const uint32_t lanes = narrow ? 8 : 32;
+  uint32_t window = narrow ? 32 : 1024;
+  while (window > lanes && groups / window * lanes < 2ull * kPackThreads * std::max(1, ctx->sm_count)) window /= 2;
+  const uint64_t threads = (groups + window - 1) / window * lanes;
+  const unsigned grid = (unsigned)((threads + kPackThreads - 1) / kPackThreads);
+  if (narrow)
+    k_pack<8><<<grid, kPackThreads, 0, ctx->stream>>>(pieces, n, g_begin, g_end, window, b->planes, b->invalid);
+  else
+    k_pack<32><<<grid, kPackThreads, 0, ctx->stream>>>(pieces, n, g_begin, g_end, window, b->planes, b->invalid);
+  launched(ctx);
+}
+
+// items (host), in the batch's order without gaps, with their device copy.  Up to 4,096 a block each, which needs no
+// search (500 reads packed in place: 32 us a call, 36 in windows); beyond that windows, since a block's warps are mostly
+// idle on a short item (200,000 reads of 251 bases from host memory: 2.36 ms a call, 3.50 with a block each).
+void launch_pack(ah_ctx* ctx, const uint8_t* d_src, const PackItem* d_items, const PackItem* items, size_t n, ah_batch* b) {
+  if (n && n <= 4096) {
+    k_pack_items<<<(unsigned)n, kPackThreads, 0, ctx->stream>>>(d_src, d_items, b->planes, b->invalid);
     launched(ctx);
+    return;
+  }
+  for (size_t i = 0; i < n; i += 0x7fffffff) {
+    const uint32_t m = (uint32_t)std::min<size_t>(0x7fffffff, n - i);
+    const PackItem& last = items[i + m - 1];
+    launch_pieces(ctx, ItemPieces{d_src, d_items + i}, m, items[i].dst_group, last.dst_group + last.n_groups, b);
   }
 }
 
-// the whole batch from records lying end to end in device memory (see k_pack_records)
+// the whole batch from records lying end to end in device memory
 void launch_pack_records(ah_ctx* ctx, const uint8_t* d_src, const uint64_t* d_rank, ah_batch* b) {
-  // 8 lanes below 16 groups a record, else 32.  Groups per window, measured: 200,000 reads of 251 bases
-  // with 64 / 32 / 16 / 8 groups 47 / 44 / 48 / 67 us; 20,011 contigs (1.20 Gbp) with 256 / 512 / 1,024 /
-  // 2,048 groups 365 / 329 / 318 / 323 us a call.  Fewer where that leaves SMs without work.
-  const bool narrow = b->n_groups < 16ull * b->n_records;
-  const uint32_t lanes = narrow ? 8 : 32;
-  uint32_t window = narrow ? 32 : 1024;
-  while (window > lanes && b->n_groups / window * lanes < 2ull * kPackThreads * std::max(1, ctx->sm_count)) window /= 2;
-  const uint64_t threads = (b->n_groups + window - 1) / window * lanes;
-  const unsigned grid = (unsigned)((threads + kPackThreads - 1) / kPackThreads);
-  if (narrow)
-    k_pack_records<8><<<grid, kPackThreads, 0, ctx->stream>>>(d_src, d_rank, b->rec_group, b->rec_len, b->n_records,
-                                                              b->n_groups, window, b->planes, b->invalid);
-  else
-    k_pack_records<32><<<grid, kPackThreads, 0, ctx->stream>>>(d_src, d_rank, b->rec_group, b->rec_len, b->n_records,
-                                                               b->n_groups, window, b->planes, b->invalid);
-  launched(ctx);
+  launch_pieces(ctx, RecordPieces{d_src, d_rank, b->rec_group, b->rec_len, b->n_groups}, b->n_records, 0, b->n_groups, b);
 }
 
 ah_status run_pack(ah_ctx* ctx, const uint8_t* d_src, const std::vector<PackItem>& items, ah_batch* b) {
@@ -323,7 +359,7 @@ ah_status run_pack(ah_ctx* ctx, const uint8_t* d_src, const std::vector<PackItem
   if (st) return st;
   AH_CUDA(ctx, cudaMemcpyAsync(d_items, items.data(), items.size() * sizeof(PackItem), cudaMemcpyHostToDevice,
                                ctx->stream));
-  launch_pack(ctx->stream, d_src, d_items, items.size(), b, ctx);
+  launch_pack(ctx, d_src, d_items, items.data(), items.size(), b);
   AH_CUDA(ctx, cudaGetLastError());
   // items (host) must stay alive until the copy has been consumed
   AH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -685,12 +721,15 @@ ah_status pack_records(ah_ctx* ctx, ah_batch* b, uint32_t first, uint32_t n, con
   };
   constexpr uint64_t kPage = 4096;
   std::vector<std::vector<Run>> runs(1);
-  std::vector<std::vector<PackItem>> items(1);
+  std::vector<PackItem> items;   // of all chunks: chunk c's are [at[c], at[c + 1])
+  std::vector<size_t> at(1, 0);
   // (220 Mbp into a plan: 1,330 us in one chunk, 1,280 this way, 1,279 to 1,300 from an eighth to a half of the rest
   // left to the last chunks and 8 to 32 MiB at least; the copy alone 1,057)
   constexpr uint64_t kLeastChunk = 16ull << 20;
   uint64_t rest = 0;  // bases not in a chunk yet
   for (uint32_t i = 0; i < n; ++i) rest += b->h_rec_len[first + i];
+  // (in one array of its final size: 200,000 reads took 0.8 ms longer with an array per chunk, joined for the upload)
+  items.reserve(n + rest / kPieceBases + 64);
   uint64_t room = kPage + next_chunk(rest, kLeastChunk, kChunkBases, 6);  // with its lead
   uint64_t fill = 0, stage_max = 0;
   const char* stretch = nullptr;  // start of the contiguous stretch of records holding record i
@@ -699,7 +738,7 @@ ah_status pack_records(ah_ctx* ctx, ah_batch* b, uint32_t first, uint32_t n, con
     const uint64_t len = b->h_rec_len[r];
     if (i == 0 || src[i] != src[i - 1] + b->h_rec_len[r - 1]) stretch = src[i];
     uint64_t done = 0;
-    if (len == 0) add_items(items.back(), b, r, 0, 0, 0);  // its padding groups (nothing is read)
+    if (len == 0) add_items(items, b, r, 0, 0, 0);  // its padding groups (nothing is read)
     while (done < len) {
       const char* sp = src[i] + done;
       uint64_t lead = 0;
@@ -712,7 +751,7 @@ ah_status pack_records(ah_ctx* ctx, ah_batch* b, uint32_t first, uint32_t n, con
       if (take < len - done) take &= ~uint64_t(31);  // split records on group boundaries
       if (take == 0) {
         runs.emplace_back();
-        items.emplace_back();
+        at.push_back(items.size());
         room = kPage + next_chunk(rest, kLeastChunk, kChunkBases, 6);
         fill = 0;
         continue;
@@ -724,20 +763,15 @@ ah_status pack_records(ah_ctx* ctx, ah_batch* b, uint32_t first, uint32_t n, con
         rv.push_back({sp - lead, take + lead, 0});
       else
         rv.push_back({sp, take, fill});
-      add_items(items.back(), b, r, done, done + take, fill);
+      add_items(items, b, r, done, done + take, fill);
       fill += take;
       rest -= take;
       stage_max = std::max(stage_max, fill);
       done += take;
     }
   }
-  std::vector<PackItem> all;
-  std::vector<size_t> at;
-  for (auto& v : items) {
-    at.push_back(all.size());
-    all.insert(all.end(), v.begin(), v.end());
-  }
-  if (all.empty()) return AH_OK;
+  at.push_back(items.size());
+  if (items.empty()) return AH_OK;
   ah_status st = AH_OK;
   uint8_t* staging[2] = {nullptr, nullptr};
   PackItem* d_items = nullptr;
@@ -746,7 +780,7 @@ ah_status pack_records(ah_ctx* ctx, ah_batch* b, uint32_t first, uint32_t n, con
   // 16 bytes of slack: the packing kernel reads whole aligned 16-byte words around its bytes
   if (!st) st = dalloc(ctx, &staging[0], stage_max + 16);
   if (!st && runs.size() > 1) st = dalloc(ctx, &staging[1], stage_max + 16);
-  if (!st) st = dalloc(ctx, &d_items, all.size());
+  if (!st) st = dalloc(ctx, &d_items, items.size());
   cudaError_t e = cudaSuccess;
   if (!st) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
   for (int k = 0; k < 2 && e == cudaSuccess && !st; ++k) {
@@ -755,7 +789,7 @@ ah_status pack_records(ah_ctx* ctx, ah_batch* b, uint32_t first, uint32_t n, con
   }
   if (!st && e == cudaSuccess) e = cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
   if (!st && e == cudaSuccess)
-    e = cudaMemcpyAsync(d_items, all.data(), all.size() * sizeof(PackItem), cudaMemcpyHostToDevice, ctx->stream);
+    e = cudaMemcpyAsync(d_items, items.data(), items.size() * sizeof(PackItem), cudaMemcpyHostToDevice, ctx->stream);
   // the staging buffers were allocated in the context stream's order: the copy stream starts after that
   if (!st && e == cudaSuccess) e = cudaEventRecord(ready, ctx->stream);
   if (!st && e == cudaSuccess) e = cudaStreamWaitEvent(cs, ready, 0);
@@ -768,13 +802,11 @@ ah_status pack_records(ah_ctx* ctx, ah_batch* b, uint32_t first, uint32_t n, con
     }
     if (e == cudaSuccess) e = cudaEventRecord(copied[w], cs);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, copied[w], 0);
-    if (e == cudaSuccess && !items[c].empty())
-      launch_pack(ctx->stream, staging[w], d_items + at[c], items[c].size(), b, ctx);
+    if (e == cudaSuccess) launch_pack(ctx, staging[w], d_items + at[c], items.data() + at[c], at[c + 1] - at[c], b);
     if (e == cudaSuccess) e = cudaEventRecord(packed[w], ctx->stream);
     if (e == cudaSuccess && on_chunk) {
-      uint64_t done = 0;
-      for (const PackItem& it : items[c]) done = std::max(done, it.dst_group + it.n_groups);
-      on_chunk(c + 1 == runs.size() ? b->n_groups : done);
+      const PackItem* last = at[c + 1] > at[c] ? &items[at[c + 1] - 1] : nullptr;
+      on_chunk(c + 1 == runs.size() ? b->n_groups : last ? last->dst_group + last->n_groups : 0);
     }
   }
   if (!st && e == cudaSuccess && !on_chunk) e = cudaStreamSynchronize(ctx->stream);
@@ -835,7 +867,7 @@ ah_status pack_concat_upto(ah_ctx* ctx, ah_batch* b, const uint8_t* d_src, const
   // pageable source: the copy is staged before the call returns, so `items` may go
   AH_CUDA(ctx, cudaMemcpyAsync(d_items, items.data(), items.size() * sizeof(PackItem), cudaMemcpyHostToDevice,
                                ctx->stream));
-  launch_pack(ctx->stream, d_src, d_items, items.size(), b, ctx);
+  launch_pack(ctx, d_src, d_items, items.data(), items.size(), b);
   AH_CUDA(ctx, cudaGetLastError());
   dfree(ctx, d_items);
   return AH_OK;
