@@ -354,11 +354,13 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
     ScanConfig win = pl->cfg;
     // the interleaved form first; where it beats the shifted form's first shape, with and without the
     // candidate queue, by a tenth (1.7x on the bench pair), the other shifted candidates, within a few
-    // percent of each other, are not tried.  Where sites are dense they are: on genomes with tandem
-    // repeats of the primers' bases one warp checks a whole repeat in the interleaved form, and the
-    // queued shifted form was up to 4 % faster (a step of 1.44 ms).
+    // percent of each other, are not tried.  Where sites are dense they are, among themselves, and the
+    // best of them meets the interleaved form at the end: on genomes with tandem repeats of the
+    // primers' bases one warp checks a whole repeat in the interleaved form, and the queued shifted
+    // form is 1 to 13 % faster (scans of 0.474 and 0.481, 0.475 and 0.544, 0.956 and 1.054 ms).
     bool shifted = true;
     int queue = pl->cfg.emit_queue;
+    const ScanConfig il = win;
     if (win.interleaved) {
       ScanConfig c = win;
       c.interleaved = 0;
@@ -369,6 +371,7 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
       }
       if (ms_q < ms * 0.97) queue = 1, ms = ms_q;
       shifted = ms < best * 1.1;
+      if (shifted) best = 1e30, win.interleaved = 0;
     }
     for (int mode = 0; mode < 2 && !st && shifted; ++mode) {
       for (auto& sh : shapes) {
@@ -395,12 +398,14 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
     // the phase split: the circuit drawn for windows surviving phase one four times as often as on
     // uniform random bases (a longer phase one) pays off on sequence whose composition lets more
     // windows through; a 1.5 % margin, the measured difference being a few percent
-    if (!st) {
+    auto longer_phase_one = [&] {
+      if (st) return;
       ScanConfig c = win;
       c.vote_windows = 4 * win.vote_windows;
       double ms = 0;
       if (!(st = time_shape(ctx, b, p, c, 2, &ms, &n_hits)) && ms < best * 0.985) best = ms, win = c;
-    }
+    };
+    longer_phase_one();
     // candidates queued per warp and emitted by the whole warp after its block: pays where sites are
     // dense (tandem repeats: the dense workload's scan went from 8.6 to 6.2 ms), costs a little
     // elsewhere (registers and shared memory)
@@ -416,6 +421,20 @@ ah_status ah_plan_create(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, co
       double ms = 0;
       if (!(st = time_shape(ctx, b, p, c, 2, &ms, &n_hits)) && (ms < best * 0.97 || prm->persistent > 0))
         best = ms, win = c;
+    }
+    // the interleaved form against the best shifted one, timed in turn, as close as they are
+    if (!st && il.interleaved && !win.interleaved) {
+      double ms_il = 0, ms_win = 0;
+      for (int round = 0; round < 2 && !st; ++round) {
+        double ms = 0, ms_w = 0;
+        if (!(st = time_shape(ctx, b, p, il, 3, &ms, &n_hits))) st = time_shape(ctx, b, p, win, 3, &ms_w, &n_hits);
+        ms_il += ms / 2, ms_win += ms_w / 2;
+      }
+      best = std::min(ms_il, ms_win);
+      if (ms_il < ms_win) {
+        win = il;
+        longer_phase_one();
+      }
     }
     pl->cfg = win;
     pl->info.best_scan_ms = best;
