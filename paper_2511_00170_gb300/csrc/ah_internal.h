@@ -352,13 +352,14 @@ void launch_scan_kernel(cudaStream_t s, const ScanKernel& k, const ah_batch* b, 
 void launch_scan_range(cudaStream_t s, const ScanKernel& k, const ah_batch* b, uint64_t* slots, uint32_t* tile_count,
                        uint32_t cap, uint32_t* status, uint64_t g0, uint64_t g1);
 // sorts every tile's keys and counts them per pair; big: n_tiles + 1 words of device scratch, used
-// when cap exceeds 256; returns the kernels launched
+// when cap exceeds 256; sites (of the sort and the emission): as many as are expected, 0 when that isn't
+// known, results do not depend on it; returns the kernels launched
 int launch_tile_sort(cudaStream_t s, uint64_t* slots, const uint32_t* tile_count, uint32_t cap, uint64_t n_tiles,
-                     uint32_t n_pairs, uint32_t* tpc, uint32_t* big, int sm_count, uint32_t* fullest);
+                     uint32_t n_pairs, uint32_t* tpc, uint32_t* big, int sm_count, uint32_t* fullest, uint64_t sites);
 void launch_emit_hits(cudaStream_t s, const uint64_t* slots, const uint32_t* tile_count, uint32_t cap, uint64_t n_tiles,
                       uint64_t tile_groups, const uint64_t* off, const ah_batch* b, ah_hit* hits,
                       const uint64_t* tile_base, uint64_t hit_cap, uint32_t* overflow, uint64_t* pair_off,
-                      uint32_t n_pairs);
+                      uint32_t n_pairs, uint64_t sites);
 void launch_pair_walk(cudaStream_t s, bool emit, const ah_hit* hits, uint64_t cap, const uint64_t* d_n,
                       const uint64_t* pair_off, const uint8_t* plen, uint32_t min_len, uint32_t max_len, uint32_t mask,
                       uint32_t* counts, const uint64_t* out_off, ah_amplicon* out, uint64_t out_cap,

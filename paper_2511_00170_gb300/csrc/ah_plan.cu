@@ -157,10 +157,10 @@ void enqueue_post(ah_plan* pl, cudaStream_t s) {
   const ah_primers* p = pl->p;
   const ah_plan_params& q = pl->prm;
   launch_tile_sort(s, pl->slots, pl->tile_count, pl->slot_cap, pl->n_tiles, p->n_pairs, pl->tpc, pl->big,
-                   pl->ctx->sm_count, pl->ctr + 0);
+                   pl->ctx->sm_count, pl->ctr + 0, pl->hit_cap);
   exclusive_scan_u32_s(s, pl->tpc, pl->tpc_off, pl->n_cells, pl->scratch);
   launch_emit_hits(s, pl->slots, pl->tile_count, pl->slot_cap, pl->n_tiles, pl->tile_groups, pl->tpc_off, b, pl->hits,
-                   nullptr, pl->hit_cap, pl->ctr + 1, pl->pair_off, p->n_pairs);
+                   nullptr, pl->hit_cap, pl->ctr + 1, pl->pair_off, p->n_pairs, pl->hit_cap);
   const uint64_t* n_hits = pl->tpc_off + pl->n_cells;
   // few sites and amplicons: one block each for the pairing and for what follows the Tm stage
   const bool few_hits = pl->hit_cap <= kOneBlockItems, few_amps = pl->amp_cap <= kOneBlockItems;

@@ -131,10 +131,13 @@ __device__ __forceinline__ void sort_tile(uint64_t* tk, uint32_t n, uint64_t t, 
 
 constexpr uint32_t kSmallTile = 256;  // keys a tile may hold to be sorted by one warp in registers
 
-// Tiles per warp of the sort and the emission: most tiles of a large batch hold no site, and a warp each only to see
-// that took longer than the work (7.6 Gbp in 232,000 tiles, 29,500 sites: 30 us each, with eight 13 and 24); fewer tiles
-// keep a warp each, so that full ones are spread.
-inline uint32_t tiles_per_warp(uint64_t n_tiles) { return n_tiles >= 65536 ? 8u : 1u; }
+// Tiles per warp of the sort and the emission.  Where most tiles of a large batch hold no site, a warp each only to see
+// that took longer than the work (7.6 Gbp in 232,000 tiles, 29,500 sites: 30 us each, with eight 13 and 24).  Fewer tiles
+// keep a warp each, and so do tiles with many sites (`sites`, as many as are expected, 0 when that isn't known), so that
+// full ones are spread: 85,000 tiles of repeats with 52 sites on average took 23 us longer with eight.
+inline uint32_t tiles_per_warp(uint64_t n_tiles, uint64_t sites) {
+  return n_tiles >= 65536 && sites < 8 * n_tiles ? 8u : 1u;
+}
 
 // A warp takes `per` tiles, one after another.  Tiles holding more keys are appended to big[1..] (count in big[0]) for
 // k_tile_sort_big.  *fullest (zero before) becomes the largest count.
@@ -485,9 +488,9 @@ void launch_scan_range(cudaStream_t s, const ScanKernel& k, const ah_batch* b, u
 // sort every tile's keys and count them per pair; `big` (n_tiles + 1 words) is needed only when
 // cap > kSmallTile
 int launch_tile_sort(cudaStream_t s, uint64_t* slots, const uint32_t* tile_count, uint32_t cap, uint64_t n_tiles,
-                     uint32_t n_pairs, uint32_t* tpc, uint32_t* big, int sm_count, uint32_t* fullest) {
+                     uint32_t n_pairs, uint32_t* tpc, uint32_t* big, int sm_count, uint32_t* fullest, uint64_t sites) {
   if (cap > kSmallTile) cudaMemsetAsync(big, 0, sizeof(uint32_t), s);
-  const uint32_t per = tiles_per_warp(n_tiles);
+  const uint32_t per = tiles_per_warp(n_tiles, sites);
   k_tile_sort<<<(unsigned)((n_tiles + 8 * per - 1) / (8 * per)), 256, 0, s>>>(slots, tile_count, cap, n_tiles, n_pairs, tpc,
                                                                               big, per, fullest);
   if (cap <= kSmallTile) return 1;
@@ -499,8 +502,8 @@ int launch_tile_sort(cudaStream_t s, uint64_t* slots, const uint32_t* tile_count
 void launch_emit_hits(cudaStream_t s, const uint64_t* slots, const uint32_t* tile_count, uint32_t cap, uint64_t n_tiles,
                       uint64_t tile_groups, const uint64_t* off, const ah_batch* b, ah_hit* hits,
                       const uint64_t* tile_base, uint64_t hit_cap, uint32_t* overflow, uint64_t* pair_off,
-                      uint32_t n_pairs) {
-  const uint32_t per = tiles_per_warp(n_tiles);
+                      uint32_t n_pairs, uint64_t sites) {
+  const uint32_t per = tiles_per_warp(n_tiles, sites);
   k_emit_hits<<<(unsigned)((n_tiles + 8 * per - 1) / (8 * per)), 256, 0, s>>>(
       slots, tile_count, cap, n_tiles, tile_groups, off, b->rec_group, b->n_records, hits, tile_base, hit_cap, overflow,
       pair_off, n_pairs, per);
@@ -737,7 +740,7 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
     cudaMemsetAsync(d_max, 0, sizeof(uint32_t), ctx->stream);
     cudaMemsetAsync(tpc, 0, n_cells * sizeof(uint32_t), ctx->stream);
     if ((st = launch_scan(ctx, b, p, cfg, per_record, tile_groups, n_tiles, slots, tile_count, cap))) return done(st);
-    launched(ctx, launch_tile_sort(ctx->stream, slots, tile_count, cap, n_tiles, n_pairs, tpc, big, ctx->sm_count, d_max));
+    launched(ctx, launch_tile_sort(ctx->stream, slots, tile_count, cap, n_tiles, n_pairs, tpc, big, ctx->sm_count, d_max, 0));
     if ((st = exclusive_scan_u32(ctx, tpc, off, n_cells))) return done(st);
     k_scan_summary<<<1, 256, 0, ctx->stream>>>(off, n_tiles, n_pairs, d_max, ctx->d_status, h->d_pair_off, ctx->h_read);
     launched(ctx);
@@ -772,7 +775,7 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
   if ((st = dalloc(ctx, &h->d, h->n))) return done(st);
   if (h->n) {
     launch_emit_hits(ctx->stream, slots, tile_count, cap, n_tiles, tile_groups, off, b, h->d, nullptr, ~0ull, nullptr,
-                     nullptr, n_pairs);
+                     nullptr, n_pairs, h->n);
     launched(ctx);
     cudaError_t e = cudaGetLastError();
     // the context's own calls are ordered after the emission; a reader on another stream waits for it
