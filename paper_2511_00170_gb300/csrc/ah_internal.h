@@ -89,7 +89,6 @@ struct ScanConfig {
                             // values weigh phase two as if windows survived phase one more often)
   int interleaved = 0;      // generated kernels: 1 the interleaved form (see ah_jit.cpp), whose tiles are
                             // kIlTileGroups groups whatever threads and groups_per_thread say
-  int il_rows = 0;          // interleaved form: positions per loop iteration (0: by the pattern count)
 };
 
 // The interleaved form: a warp takes kIlTileGroups consecutive groups, a block kIlWarps of them.

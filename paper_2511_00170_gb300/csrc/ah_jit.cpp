@@ -886,13 +886,20 @@ static __device__ __forceinline__ void push4(u32 c0, u32 c1, u32 c2, u32 c3, int
 // registers and the loop body the instruction cache.  1.92 Gbp of random bases, 8 / 4 / 2 positions:
 // one pair 0.290 / 0.320 ms, two pairs 0.440 / 0.460, four pairs 0.802 / 0.755 / 0.852, eight pairs
 // 1.480 / 1.132 / 1.228.
-int il_rows(int patterns) { return patterns <= 8 ? 8 : patterns <= 32 ? 4 : 2; }
+// At most so many that a lane's words of an iteration fit the queue: one that overflows it is run again
+// for as many lanes at a time as the queue holds, at least one.
+int il_rows(int patterns) {
+  int rows = patterns <= 8 ? 8 : patterns <= 32 ? 4 : 2;
+  while (rows > 1 && rows * ((patterns + 3) / 4) > kIlQueue) rows /= 2;
+  return rows;
+}
 // Blocks per SM the registers must allow (shared memory holds six): at six the compiler takes up to 168
 // registers; one pair needs fewer and ran 4 % faster bounded for seven.
 int il_blocks(int patterns) { return patterns <= 4 ? 7 : 6; }
 
 std::string interleaved_source(const std::vector<Pattern>& pats, const ScanConfig& cfg, int* alu_ops_per_group) {
-  const int Q = (int)pats.size(), R = cfg.il_rows > 0 ? cfg.il_rows : il_rows(Q);
+  const int Q = (int)pats.size(), R = il_rows(Q);
+  if (R * ((Q + 3) / 4) > kIlQueue) return "#error more patterns than the interleaved form's queue holds\n";
   std::ostringstream os;
   os << "// generated scan kernel, interleaved form: " << Q << " patterns\n";
   os << "#define NT " << 32 * kIlWarps << "\n#define QCAP " << kIlQueue << "\n";
@@ -1280,7 +1287,7 @@ std::string kernel_key(int device, const std::vector<Pattern>& pats, const ScanC
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, device);
   const int32_t f[] = {major * 10 + minor, cfg.threads,    cfg.groups_per_thread, cfg.shift_mode,  cfg.persistent,
-                       cfg.min_blocks,     cfg.emit_queue, cfg.vote_windows,      cfg.interleaved, cfg.il_rows};
+                       cfg.min_blocks,     cfg.emit_queue, cfg.vote_windows,      cfg.interleaved};
   std::string key((const char*)f, sizeof f);
   for (const Pattern& P : pats) {
     const uint8_t h[] = {P.len, P.clamp_lo, P.clamp_hi, P.k, (uint8_t)(P.id & 255), (uint8_t)(P.id >> 8)};

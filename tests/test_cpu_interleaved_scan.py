@@ -166,3 +166,13 @@ def test_self_check(dump, tmp_path, k, primers, clamp):
     rc, status, _, sites = run(build(str(tmp_path), src.replace(m.group(0), f"const u32 f1_1 = {m.group(1)} & ~2u;")),
                                str(tmp_path), text)
     assert (rc, status) == (0, 1) and sites == want
+
+
+def test_more_patterns_than_an_iteration_may_queue(dump, tmp_path):
+    """Sets far above what plans give the form (128 patterns): the iteration shrinks so that the queue holds one lane's
+    words at least, and a set that cannot fit is refused when the kernel is built, not left to spin."""
+    many = [synth.random_primer(synth.Stream(synth.make_key(5, i, 0)), 12, 2, 0) for i in range(100)]   # 200 patterns
+    text = _repeats(33_000, 3, many[:2], 0.1)
+    rc, status, _, sites = run(build(str(tmp_path), dump("source", 0, 1, many)), str(tmp_path), text, order=2)
+    assert (rc, status) == (0, 0) and sites == expected(text, many, 0, 1) and len(sites) > 100
+    assert dump("compile", 0, 1, many * 2).startswith("error")   # 400 patterns
