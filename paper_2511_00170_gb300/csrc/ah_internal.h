@@ -101,6 +101,17 @@ inline uint64_t scan_block_groups(const ScanConfig& c) {
   return c.interleaved ? (uint64_t)kIlTileGroups * kIlWarps : (uint64_t)c.threads * c.groups_per_thread;
 }
 
+// The generic scan kernel's blocks for `groups` groups, each block threads * groups_per_thread of them whatever
+// the slot lists' tiles are, and the tiles that one launch's grid can cover.
+inline uint64_t generic_blocks(const ScanConfig& c, uint64_t groups) {
+  const uint64_t per = (uint64_t)c.threads * c.groups_per_thread;
+  return (groups + per - 1) / per;
+}
+inline uint64_t generic_tiles_per_launch(const ScanConfig& c) {
+  const uint64_t per = (uint64_t)c.threads * c.groups_per_thread;
+  return std::max<uint64_t>(1, 0x7fffffffull * per / scan_tile_groups(c));
+}
+
 // default of ah_ctx::tm_split_sites: each launch re-reads the window's site marks, which pays once
 // the chains of fewer primers per launch keep the instruction cache warm
 constexpr uint64_t kTmSplitSitesDefault = 4ull << 20;

@@ -385,8 +385,8 @@ __device__ __noinline__ void gen_emit(uint32_t h, const GenPattern& P, uint64_t 
   }
 }
 
-// one CTA per tile of blockDim.x * gpt groups (the tiles of the slot lists); the pattern table is
-// staged in shared memory; every thread takes gpt groups and tests each against every pattern
+// one CTA per blockDim.x * gpt groups (a tile of the slot lists is one such piece, or kIlTileGroups groups
+// where a plan's sizing run has the interleaved form's tiles); the pattern table is staged in shared memory; every thread takes gpt groups and tests each against every pattern
 __global__ void k_scan_generic(const uint2* __restrict__ planes, const uint32_t* __restrict__ invalid,
                                uint64_t group_begin, uint64_t n_groups, const GenPattern* __restrict__ pats,
                                int n_pats, int gpt, uint64_t tile_groups, uint64_t* __restrict__ slots,
@@ -522,12 +522,12 @@ ah_status enqueue_generic(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, c
   const size_t Q = p->pats.size();
   for (size_t q0 = 0; q0 < Q; q0 += kGenMaxPatterns) {
     const int nq = (int)std::min<size_t>(kGenMaxPatterns, Q - q0);
-    for (uint64_t t0 = t_begin; t0 < t_end; t0 += 0x7fffffffull) {
-      const uint64_t nt = std::min<uint64_t>(0x7fffffffull, t_end - t0);
+    for (uint64_t t0 = t_begin, nt; t0 < t_end; t0 += nt) {
+      nt = std::min(generic_tiles_per_launch(cfg), t_end - t0);
       const uint64_t g0 = t0 * tile_groups;
       const uint64_t ng = std::min<uint64_t>(b->n_groups - std::min(b->n_groups, g0), nt * tile_groups);
       if (ng == 0) continue;
-      k_scan_generic<<<(unsigned)nt, cfg.threads, nq * sizeof(GenPattern), ctx->stream>>>(
+      k_scan_generic<<<(unsigned)generic_blocks(cfg, ng), cfg.threads, nq * sizeof(GenPattern), ctx->stream>>>(
           b->planes, b->invalid, g0, ng, p->d_gen + q0, nq, cfg.groups_per_thread, tile_groups, slots, tile_count, cap,
           ctx->d_status);
       const cudaError_t le = cudaGetLastError();

@@ -2,6 +2,8 @@
 // usage: il_dump source|compile|ops|suits [windows=N] k clamp primer [primer ...]
 // (each primer gives its + and - strand patterns and may carry its own budget as "PRIMER:k"; "compile" compiles for
 // sm_103a with NVRTC, no device needed; "suits" prints whether plans choose the form for these patterns)
+//        il_dump generic threads groups_per_thread tiles
+// (the groups that the generic kernel's blocks cover for so many of the form's tiles, and those of a full launch)
 #define main jit_dump_main
 #include "jit_dump.cpp"
 #undef main
@@ -13,6 +15,14 @@ int main(int argc, char** argv) {
   int a = 2;
   ah::ScanConfig cfg;
   cfg.interleaved = 1;
+  if (what == "generic") {
+    cfg.threads = atoi(argv[2]), cfg.groups_per_thread = atoi(argv[3]);
+    const unsigned long long per = 1ull * cfg.threads * cfg.groups_per_thread, tile = ah::scan_tile_groups(cfg);
+    const unsigned long long most = ah::generic_tiles_per_launch(cfg);
+    printf("%llu %llu %llu\n", (unsigned long long)ah::generic_blocks(cfg, atoll(argv[4]) * tile) * per, most,
+           (unsigned long long)ah::generic_blocks(cfg, most * tile));
+    return 0;
+  }
   if (!strncmp(argv[a], "windows=", 8)) cfg.vote_windows = atoi(argv[a++] + 8);
   const int k = atoi(argv[a]), clamp = atoi(argv[a + 1]);
   std::vector<ah::Pattern> pats;

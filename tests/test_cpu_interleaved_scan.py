@@ -176,3 +176,14 @@ def test_more_patterns_than_an_iteration_may_queue(dump, tmp_path):
     rc, status, _, sites = run(build(str(tmp_path), dump("source", 0, 1, many)), str(tmp_path), text, order=2)
     assert (rc, status) == (0, 0) and sites == expected(text, many, 0, 1) and len(sites) > 100
     assert dump("compile", 0, 1, many * 2).startswith("error")   # 400 patterns
+
+
+@pytest.mark.parametrize("threads,groups", [(32, 1), (64, 4), (128, 8), (256, 4), (256, 8), (1024, 16), (96, 5)])
+def test_generic_kernel_covers_the_forms_tiles(dump, threads, groups):
+    """The generic kernel, which scans first on contexts that compile in the background, has blocks enough for every
+    group of the interleaved form's tiles whatever the context's scan shape, and grids within the limit."""
+    exe = os.path.join(BUILD, "il_dump")
+    for tiles in (1, 2, 511, 100_003):
+        covered, most, blocks = map(int, subprocess.check_output([exe, "generic", str(threads), str(groups), str(tiles)]).split())
+        assert tiles * 1024 <= covered < tiles * 1024 + threads * groups
+        assert most >= 1 and blocks <= 0x7fffffff

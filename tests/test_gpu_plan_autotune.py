@@ -51,3 +51,39 @@ def test_form_and_results(engine, n, repeats):
         assert len(ref.hits) > 50_000
     elif n > 100_000_000:
         assert interleaved, info
+
+
+@pytest.mark.parametrize("mode", [1, 2, 3])
+def test_interleaved_plan_on_a_context_with_the_generic_scan(engine, mode):
+    """Contexts that scan with the generic kernel, first or throughout: a plan of the interleaved form is sized over that
+    form's tiles by it, and finds what the regular path finds."""
+    from paper_2511_00170_gb300 import ah
+    from paper_2511_00170_gb300.pipeline import Engine, Params
+
+    n = 20_000_000
+    seq = np.frombuffer(b"ACGT", np.uint8)[np.random.default_rng(mode).integers(0, 4, n, dtype=np.uint8)]
+    wl = synth.random_small(3, n_records=1, len_lo=10, len_hi=10, n_pairs=1, plant=0)
+    wl.fwd, wl.rev, wl.k, wl.clamp = ["ACGTTGCAAG" + "ACG"[mode - 1]], ["TTGACRSTAGC"], [1], 2
+    wl.min_len, wl.max_len, wl.tm.min_tm = 20, 4000, None
+    p = Params.from_workload(wl)
+    off = np.array([0, n], dtype=np.int64)
+    batch = engine.pack(seq, off)
+    e = Engine(0)
+    try:
+        ref = engine.step(batch, p)
+        ah.ah_ctx_set_generic_scan(e.ctx, mode)
+        mine = e.pack(seq, off)
+        plan = e.plan(mine, p)
+        try:
+            info = ah.ah_plan_info_get(plan)
+            assert (info["threads"], info["groups_per_thread"]) == (64, 32)
+            ah.ah_plan_run(plan, e.ctx)
+            out = e.plan_output(plan)
+        finally:
+            ah.ah_plan_free(plan)
+            ah.ah_batch_free(mine)
+    finally:
+        e.close()
+        ah.ah_batch_free(batch)
+    assert len(ref.hits) > 100
+    assert out.hits.tobytes() == ref.hits.tobytes() and out.amps.tobytes() == ref.amps.tobytes() and out.arena == ref.arena
