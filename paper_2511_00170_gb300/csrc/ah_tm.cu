@@ -839,8 +839,14 @@ __device__ __forceinline__ int nth_choice(uint32_t ch, uint32_t n) {
 // and a variant's Tm is the walk's (enum_max), so the maximum is the same number.
 //
 // FP64 runs at a sixteenth of a warp instruction per cycle, so a variant is evaluated in single
-// precision first and skipped when that lies 0.05 K below the best so far: with |dS| above 50 and
-// temperatures below 2,000 K rounding moves it by 3e-6 of itself, 0.006 K, at most.
+// precision first and skipped when that lies 0.05 K below the best so far; the maximum itself is always
+// an FP64 evaluation.  The screen is used only where rounding (u = 6e-8 a step) cannot move it so far:
+// with dS < -50 the sums' terms cancel to no less than half their magnitudes, so the temperature before
+// the salt correction, T0 = dH / dS in 200 to 500 K, is off by 13 u T0 and 6 u 800 K, 1e-3 K together; the
+// correction 1/T = 1/T0 + c takes that to (T / T0)^2 <= 6.25 times as much, 0.006 K with T in 200 to 500 K
+// too, and adds T^2 times the rounding of c and of the sum, 5 u (|c0| + |c1| + |c2|) + 3 u / 200, which
+// is 0.019 + 0.0003 K for coefficients that add up to less than 0.25: 0.026 K in all.  (At 10 uM to 1 M of
+// salt they add up to less than 0.03.)
 // With one lane walking a site's variants position by position, ah_tm_filter took 2,202 us for the
 // 6,200 sites of four pairs (up to 128 combinations each) on 60 Mbp of contigs; with this 296 us.
 constexpr uint32_t kTmGroupEnum = 2048;  // combinations; sites with more keep the walk, which prunes
@@ -848,6 +854,7 @@ template <int G>
 __device__ double group_enum_max(const TmGroupSh& sh, const int32_t* __restrict__ w, int D, uint32_t combos, int K,
                                  int m0, int gc0, int L, const TmRun& R, int r, unsigned gmask) {
   const float h0 = (float)R.init_h, s0 = (float)(R.init_s + R.sym_s + R.rlnk), h1 = (float)R.sym_h;
+  const bool mild = fabs(R.rc0) + fabs(R.rc1) + fabs(R.rc2) < 0.25;
   double best = -INFINITY;
   bool any = false;
   for (uint32_t x = (uint32_t)r; x < combos; x += G) {
@@ -873,10 +880,10 @@ __device__ double group_enum_max(const TmGroupSh& sh, const int32_t* __restrict_
     const float dh = 0.1f * (float)dh10 + h0 + h1 + (float)(gc ? R.onegc_h : R.allat_h);
     const float ds = 0.1f * (float)ds10 + s0 + (float)(gc ? R.onegc_s : R.allat_s);
     const float tk = 1000.f * dh / ds;
-    if (ds < -50.f && fabsf(tk) < 2000.f) {
+    if (mild && ds < -50.f && tk > 200.f && tk < 500.f) {
       const float corr = (float)R.rc0 + (float)R.rc1 * ((float)gc / (float)L) + (float)R.rc2 / (2.f * (float)(L - 1));
       const float inv = 1.f / tk + corr;
-      if (fabsf(inv) > 5e-4f && 1.f / inv - 273.15f < (float)best - 0.05f) continue;
+      if (inv > 2e-3f && inv < 5e-3f && 1.f / inv - 273.15f < (float)best - 0.05f) continue;
     }
     best = fmax(best, tm_of_tenths(dh10, ds10, gc, L, R));
   }
