@@ -187,3 +187,74 @@ def test_generic_kernel_covers_the_forms_tiles(dump, threads, groups):
         covered, most, blocks = map(int, subprocess.check_output([exe, "generic", str(threads), str(groups), str(tiles)]).split())
         assert tiles * 1024 <= covered < tiles * 1024 + threads * groups
         assert most >= 1 and blocks <= 0x7fffffff
+
+
+TILE = 32768
+
+
+@pytest.mark.parametrize("k,clamp,primers", [
+    (2, 3, PLAIN), (0, 0, ["ACGTACGT"]), (1, 2, ["ACGRYSWKMBDHVN"]), (3, 3, ["NNNNACGTNNNNACGTAC"]),
+    (5, 1, ["ACGTAGCTAGCTAGCATCGATCGATCGATCGA"]), (7, 0, ["AGCTTGACCGTAGGCATTAC"]), (2, 20, ["AGCTTGACCGTAGGCATTAC"]),
+    (6, 3, ["RRRRRRRRRRYYYYYYYYYY"]), (0, 2, ["AC"]), (0, 0, EIGHT), (1, 3, [f"{p}:{i % 4}" for i, p in enumerate(EIGHT)]),
+    (3, 3, EIGHT + PLAIN + [p[::-1] for p in EIGHT])])
+def test_sites_equal_the_exact_count(dump, tmp_path, k, clamp, primers):
+    """Every set's sites on random bases with planted copies, invalid bases, and windows over every kind of edge: a
+    group's, a lane's (the next lane's words), a tile's and the batch's."""
+    exe = build(str(tmp_path), dump("source", k, clamp, primers))
+    rng = np.random.default_rng(len(primers) + k)
+    text = list(_random(2 * TILE + 77, k))
+    first = primers[0].split(":")[0]
+    for at in (0, 31, 1000, 1023, 1024, TILE - 40, TILE - 32, TILE - 19, TILE - 1, TILE, 2 * TILE - 5, 2 * TILE + 77 - len(first)):
+        p = primers[int(rng.integers(len(primers)))].split(":")[0] if at % 2 else first
+        if at + len(p) <= len(text):
+            text[at:at + len(p)] = [SETS[c][int(rng.integers(len(SETS[c])))] for c in p]
+    for at in rng.integers(0, len(text), 40):
+        text[at] = "N"
+    text = "".join(text)
+    want = expected(text, primers, k, clamp)
+    for order in (0, 2):
+        rc, status, counts, sites = run(exe, str(tmp_path), text, order=order)
+        assert (rc, status) == (0, 0) and sites == want
+    # a range of tiles, as an upload scans it: what starts in it, and nothing else
+    rc, status, _, sites = run(exe, str(tmp_path), text, first=1024, count=1024)
+    assert (rc, status) == (0, 0) and sites == [s for s in want if s[0] == 1]
+    # slot lists shorter than a tile's sites: counted in full, the lists hold what fits
+    rc, _, counts, _ = run(exe, str(tmp_path), text, cap=1)
+    assert rc == 0 and counts.sum() == len(want)
+
+
+@pytest.mark.parametrize("n", [1, 9, 31, 32, 33, 63, 65, 1000, TILE - 1, TILE, TILE + 1, TILE + 33])
+def test_sizes(dump, tmp_path, n):
+    exe = build(str(tmp_path), dump("source", 1, 1, ["ACGT", "GGA"]))
+    text = _random(n, n)
+    rc, status, _, sites = run(exe, str(tmp_path), text, order=3)
+    assert (rc, status) == (0, 0) and sites == expected(text, ["ACGT", "GGA"], 1, 1)
+
+
+@pytest.mark.parametrize("windows", [1024, 4096])
+@pytest.mark.parametrize("primers", [PLAIN, EIGHT, EIGHT * 4], ids=["one pair", "eight", "thirty-two"])
+def test_compiles(dump, primers, windows):
+    """For sm_103a, with NVRTC on the host: the smallest and the largest set that plans give the form, at the phase splits
+    that the autotuner tries."""
+    out = dump("compile", 2, 3, primers, windows=windows)
+    assert out.startswith("compiled "), out[:2000]
+
+
+def test_which_sets_suit(dump):
+    """Plans choose the form for sets whose filters leave few windows, of at most 32 pairs."""
+    assert dump("suits", 3, 3, PLAIN).strip() == "1" and dump("suits", 2, 3, EIGHT * 4).strip() == "1"
+    assert dump("suits", 0, 0, ["AC"]).strip() == "0" and dump("suits", 1, 0, ["NN"]).strip() == "0"
+    assert dump("suits", 2, 3, EIGHT * 4 + PLAIN).strip() == "0"
+
+
+def test_bench_tables_describe_the_generated_circuits(dump):
+    """bench.py keys its measured ALU-pipe and DRAM figures of this form by circuit size: the bench pair's 71 instructions
+    per 32 positions and the 8-pair batched set's 324, k = i mod 4."""
+    import bench
+
+    assert int(dump("ops", 3, 3, PLAIN)) == 71
+    wl = synth.batched(n_genomes=3)
+    batched = [f"{p}:{k}" for f, r, k in zip(wl.fwd, wl.rev, wl.k) for p in (f, r)]
+    assert int(dump("ops", 0, wl.clamp, batched)) == 324
+    for ops in (71, 324):
+        assert ops in bench.SCAN_PIPE and (ops, 64, 32, 0, 0) in bench.SCAN_TRAFFIC
