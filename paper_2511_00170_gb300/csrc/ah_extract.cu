@@ -126,7 +126,7 @@ __device__ __forceinline__ uint4 unit_letters(const UnitBits& x) {
 // lane and step took 147, sixteen lanes per amplicon and a unit per lane 107 (most of it spent on the fields, once
 // per lane).
 constexpr int kExThreads = 128, kExAmps = 32, kExMinAmps = 4;
-constexpr uint64_t kExBlocks = 152 * 16;
+constexpr uint64_t kExBlocksPerSm = 16;
 
 __global__ void __launch_bounds__(kExThreads) k_extract_write(
     const ah_amplicon* __restrict__ amps, uint64_t n, const ah_hit* __restrict__ hits, const uint2* __restrict__ planes,
@@ -197,7 +197,10 @@ __global__ void __launch_bounds__(kExThreads) k_extract_write(
   }
 }
 
-unsigned extract_blocks(uint64_t n) { return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(kExBlocks, (n + kExMinAmps - 1) / kExMinAmps)); }
+unsigned extract_blocks(uint64_t n, int sm_count) {
+  const uint64_t most = kExBlocksPerSm * (uint64_t)std::max(1, sm_count);
+  return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(most, (n + kExMinAmps - 1) / kExMinAmps));
+}
 
 // What follows the Tm stage in one block for up to kOneBlockItems amplicons: threshold, compaction (with the filter) and,
 // with ebase, the bytes of each kept amplicon and their offsets.  4 kept of 26 amplicons took 36 us in nine kernels, 7.4
@@ -282,13 +285,13 @@ void launch_finish_one(cudaStream_t s, ah_amplicon* amps, uint64_t cap, const ui
 void launch_extract(cudaStream_t s, bool write, const ah_amplicon* amps, uint64_t cap, const uint64_t* d_n,
                     const ah_hit* hits, const uint2* planes, const uint32_t* invalid, const uint64_t* rec_group,
                     const uint32_t* rec_len, const uint8_t* plen, int trim, uint32_t fb, uint32_t rb, uint64_t* len_or_base,
-                    char* arena, uint64_t* field_off, uint64_t arena_cap, uint32_t* overflow) {
+                    char* arena, uint64_t* field_off, uint64_t arena_cap, uint32_t* overflow, int sm_count) {
   if (!write)
     k_extract_len<<<(unsigned)std::max<uint64_t>(1, (cap + 255) / 256), 256, 0, s>>>(amps, cap, hits, rec_len, plen, trim,
                                                                                     (int64_t)fb, (int64_t)rb,
                                                                                     len_or_base, d_n);
   else
-    k_extract_write<<<extract_blocks(cap), kExThreads, 0, s>>>(
+    k_extract_write<<<extract_blocks(cap, sm_count), kExThreads, 0, s>>>(
         amps, cap, hits, planes, invalid, rec_group, rec_len, plen, trim, (int64_t)fb, (int64_t)rb, len_or_base, arena,
         field_off, d_n, arena_cap, overflow);
 }
@@ -313,7 +316,7 @@ ah_status extract(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, const ah_
   const uint64_t bytes = ctx->h_read[0];
   if ((st = dalloc(ctx, &a->d_arena, bytes)) || (st = dalloc(ctx, &a->d_field_off, 5 * n + 1))) return st;
   if (n) {
-    k_extract_write<<<extract_blocks(n), kExThreads, 0, ctx->stream>>>(a->d, n, h->d, b->planes, b->invalid, b->rec_group,
+    k_extract_write<<<extract_blocks(n, ctx->sm_count), kExThreads, 0, ctx->stream>>>(a->d, n, h->d, b->planes, b->invalid, b->rec_group,
                                                                      b->rec_len, p->d_plen, trim, (int64_t)fb,
                                                                      (int64_t)rb, base, a->d_arena, a->d_field_off);
     launched(ctx);

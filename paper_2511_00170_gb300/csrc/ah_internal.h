@@ -276,10 +276,8 @@ constexpr uint64_t kBounceBytes = 8ull << 20;  // each of a context's two bounce
 // both bounce buffers allocated, and no upload from the first in flight
 ah_status stage_buffer(ah_ctx* ctx);
 constexpr int kReadWords = 512;  // page-locked words of a context for counts read back
-// read one uint64 (or n of them, at most 8, from places of their own) from device memory through the
-// context's page-locked words, in one synchronisation of the stream
+// read one uint64 from device memory through the context's page-locked words (synchronises the stream)
 ah_status read_u64(ah_ctx* ctx, const uint64_t* d, uint64_t* h);
-ah_status read_u64s(ah_ctx* ctx, int n, const uint64_t* const* d, uint64_t* const* h);
 // ah_pack_batch_device without its wait: d_seq must stay until ctx->stream has passed the packing.
 ah_status pack_device_records(ah_ctx* ctx, uint32_t n_rec, const uint8_t* d_seq, const uint64_t* h_offsets,
                               const uint32_t* genome_ids, ah_batch** out);
@@ -422,7 +420,7 @@ void launch_compact_amps(cudaStream_t s, const ah_amplicon* in, uint64_t cap, co
 void launch_extract(cudaStream_t s, bool write, const ah_amplicon* amps, uint64_t cap, const uint64_t* d_n,
                     const ah_hit* hits, const uint2* planes, const uint32_t* invalid, const uint64_t* rec_group,
                     const uint32_t* rec_len, const uint8_t* plen, int trim, uint32_t fb, uint32_t rb, uint64_t* len_or_base,
-                    char* arena, uint64_t* field_off, uint64_t arena_cap, uint32_t* overflow);
+                    char* arena, uint64_t* field_off, uint64_t arena_cap, uint32_t* overflow, int sm_count);
 
 // ---- run-time specialised scan kernels (ah_jit.cpp) ------------------------------------------
 struct ScanKernel {

@@ -193,7 +193,8 @@ void enqueue_post(ah_plan* pl, cudaStream_t s) {
   }
   if (q.extract && !few_amps) {
     launch_extract(s, false, out, pl->amp_cap, n_out, pl->hits, b->planes, b->invalid, b->rec_group, b->rec_len,
-                   p->d_plen, q.trim, q.fb_len, q.rb_len, pl->elen, nullptr, nullptr, 0, nullptr);
+                   p->d_plen, q.trim, q.fb_len, q.rb_len, pl->elen, nullptr, nullptr, 0, nullptr,
+                   pl->ctx->sm_count);
     exclusive_scan_u64_s(s, pl->elen, pl->ebase, pl->amp_cap, pl->scratch);
   }
   // the counters are all there: written to the host beside the extraction, on a branch of the graph (a 30 Mbp replay with
@@ -210,7 +211,7 @@ void enqueue_post(ah_plan* pl, cudaStream_t s) {
   if (q.extract)
     launch_extract(s, true, out, pl->amp_cap, n_out, pl->hits, b->planes, b->invalid, b->rec_group, b->rec_len,
                    p->d_plen, q.trim, q.fb_len, q.rb_len, pl->ebase, pl->arena, pl->field_off, pl->arena_cap,
-                   pl->ctr + 1);
+                   pl->ctr + 1, pl->ctx->sm_count);
   if (branch) cudaStreamWaitEvent(s, pl->join, 0);
 }
 

@@ -71,15 +71,9 @@ ah_status copy_to_host(ah_ctx* ctx, void* dst, const void* src, uint64_t bytes) 
 }
 
 ah_status read_u64(ah_ctx* ctx, const uint64_t* d, uint64_t* h) {
-  return read_u64s(ctx, 1, &d, &h);
-}
-
-ah_status read_u64s(ah_ctx* ctx, int n, const uint64_t* const* d, uint64_t* const* h) {
-  if (n > 8) return fail(ctx, AH_EINTERNAL, "read_u64s: %d values", n);
-  for (int i = 0; i < n; ++i)
-    AH_CUDA(ctx, cudaMemcpyAsync(ctx->h_read + i, d[i], sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
+  AH_CUDA(ctx, cudaMemcpyAsync(ctx->h_read, d, sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
   AH_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  for (int i = 0; i < n; ++i) *h[i] = ctx->h_read[i];
+  *h = ctx->h_read[0];
   return AH_OK;
 }
 
