@@ -1868,9 +1868,11 @@ int launch_tm_hits(cudaStream_t s, const TmRun& R, const ah_primers* p, const ah
     // of eight pairs 69 -> 26, 344,000 slots of reads 75 -> 50, 83,000 to 614,000 slots of repeats 82 -> 30 to 124 -> 98
     // (937,000, windows of 1,024 either way: 147).  Every block also fills its tables, so windows that make
     // more blocks than the SMs hold at once (eight each) lose: 2.8 million slots of repeats take 372 us in windows of
-    // 1,024, 442 of 512 and 868 of 128.
+    // 1,024, 442 of 512 and 868 of 128.  Under salt methods 6 and 7 every site is listed for k_tm_deferred and there is no
+    // chain to share out: large windows, which list the sites of a primer together (458,616 sites of repeats 20.0 ms,
+    // 20.5 in windows of 512).
     int window = kTmSlots;
-    while (window > kTmThreads && cap < 4ull * (uint64_t)std::max(1, sm_count) * (uint64_t)window) window /= 2;
+    while (R.saltcorr < 6 && window > kTmThreads && cap < 4ull * (uint64_t)std::max(1, sm_count) * (uint64_t)window) window /= 2;
     const unsigned grid = (unsigned)std::max<uint64_t>(1, (cap + window - 1) / window);
     const size_t smem_j = 4 * ((size_t)kTmThreadFixedWords + (size_t)tk.weight_words * kTmThreads);
     if (tk.fn && tk.image && smem_j <= kTmSmemCap) {  // the kernel generated for this primer set
