@@ -133,10 +133,11 @@ constexpr uint32_t kSmallTile = 256;  // keys a tile may hold to be sorted by on
 
 // Tiles per warp of the sort and the emission.  Where most tiles of a large batch hold no site, a warp each only to see
 // that took longer than the work (7.6 Gbp in 232,000 tiles, 29,500 sites: 30 us each, with eight 13 and 24).  Fewer tiles
-// keep a warp each, and so do tiles with many sites (`sites`, as many as are expected, 0 when that isn't known), so that
-// full ones are spread: 85,000 tiles of repeats with 52 sites on average took 23 us longer with eight.
+// keep a warp each, so that full ones are spread; where tiles hold many sites on average (`sites`, as many as are expected, 0
+// when that isn't known) it takes more tiles until a block's share evens out: with 52 sites per tile 85,000 tiles took 23 us
+// longer with eight, 170,000 as long, and 578,000 (18.9 Gbp) 140 us less.
 inline uint32_t tiles_per_warp(uint64_t n_tiles, uint64_t sites) {
-  return n_tiles >= 65536 && sites < 8 * n_tiles ? 8u : 1u;
+  return n_tiles >= (sites < 8 * n_tiles ? 65536u : 262144u) ? 8u : 1u;
 }
 
 // A warp takes `per` tiles, one after another.  Tiles holding more keys are appended to big[1..] (count in big[0]) for
