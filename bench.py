@@ -409,7 +409,7 @@ def e2e_from_fasta(ah, eng, wl, batch, plan, bufs, on_device, steps):
     del t_text
     return {"value": wl.total_bp / t_overlap / 1e9, "unit": "Gbp/s", "h2d_bytes_per_step": n,
             "ms_per_step": t_overlap * 1e3,
-            "path": "pinned FASTA text (80-column lines) -> ah_plan_launch_fasta (parsed on the device in 256 MiB "
+            "path": "pinned FASTA text (80-column lines) -> ah_plan_launch_fasta (parsed on the device in "
                     "chunks as they land, completed records packed and their tiles scanned at once) -> "
                     "ah_plan_copy_results into pinned host buffers",
             "parse_then_step": {"value": wl.total_bp / t_serial / 1e9, "unit": "Gbp/s", "ms_per_step": t_serial * 1e3,
@@ -507,7 +507,7 @@ def run_engine(args):
     roofline["step_gbps_frac_of_alu_bound"] = value / world / (ALU_PEAK_TOPS * 1e3 / roofline["circuit"]["ops_per_base"])
 
     # end to end through the C ABI from pinned host memory: every step packs the records from host
-    # ASCII into the plan's batch (copy engines in 256 Mi-base chunks, packed from HBM as they land),
+    # ASCII into the plan's batch (copy engines in chunks of up to 256 Mi bases, packed from HBM as they land),
     # replays the plan and copies sites, amplicons and sequences into pinned host buffers
     e2e = None
     if not args.no_e2e:
@@ -595,7 +595,7 @@ def run_engine(args):
             "h2d_bytes_per_step": planes.nbytes + groups.nbytes + words.nbytes, "d2h_bytes_per_step": d2h,
             "ms_per_step": t_overlap * 1e3,
             "path": "pinned 2-bit planes + sparse invalid words -> ah_plan_launch_packed (invalid words first, "
-                    "planes in 256 Mi-base chunks, each range of scan tiles scanned as its planes land) -> "
+                    "planes in chunks of up to 256 Mi bases, each range of scan tiles scanned as its planes land) -> "
                     "ah_plan_copy_results into pinned host buffers",
             "import_then_step": {"value": wl.total_bp / t_serial / 1e9, "unit": "Gbp/s", "ms_per_step": t_serial * 1e3,
                                  "path": "ah_batch_import -> ah_plan_launch -> ah_plan_copy_results"}}

@@ -204,9 +204,9 @@ typedef struct {
 
 /* Pack host ASCII records.  seqs[i] points at lens[i] characters (no terminator needed);
  * genome_ids may be NULL (then record i has genome id i).  Characters other than ACGTacgt are
- * invalid bases.  Records are copied to the device by the copy engines in chunks of up to 256 Mi
- * bases (64 MB packed), one copy per run of records contiguous in host memory, on a second stream,
- * and each chunk is packed from device memory while the next one is in flight; page-locked host
+ * invalid bases.  Records are copied to the device by the copy engines in chunks of three quarters of
+ * what is left (16 to 256 Mi bases), one copy per run of records contiguous in host memory, on a second
+ * stream, and each chunk is packed from device memory while the next one is in flight; page-locked host
  * memory (cudaHostAlloc, cudaHostRegister, pinned tensors) moves at the full host-link rate.
  * Records already in device memory are packed in place.  Synchronises the stream before
  * returning (the host buffers may be reused afterwards).  AH_EINVAL: n_rec == 0, a record longer
@@ -262,7 +262,7 @@ void ah_fasta_free(ah_fasta* f);
 
 /* Pack records that are already in device memory: d_seq holds all records back to back and
  * h_offsets (host, n_rec+1 entries) gives record r as d_seq[h_offsets[r], h_offsets[r+1]).
- * Asynchronous; d_seq must stay valid until the stream reaches this work. */
+ * Synchronises the stream before returning (d_seq may be reused afterwards). */
 ah_status ah_pack_batch_device(ah_ctx* ctx, uint32_t n_rec, const uint8_t* d_seq, const uint64_t* h_offsets,
                                const uint32_t* genome_ids, ah_batch** out);
 
@@ -568,9 +568,9 @@ ah_status ah_plan_launch_host(ah_plan* plan, const uint8_t* h_seq, const uint64_
 /* The step on genomes stored as 2-bit batches in host memory (the layout ah_batch_export writes for
  * the plan's batch: planes, n_invalid sparse invalid words at groups inv_groups; Abstract and Section
  * "Implementations": AHv2 streams 2-bit batches): the invalid words are written first, then the
- * planes cross the link in chunks of 256 Mi bases straight into the batch, and each range of scan
- * tiles whose groups (and the group after them) have landed is scanned while the next chunk is
- * copied; the rest of the step follows as one graph launch.  Results as after ah_plan_launch.
+ * planes cross the link in chunks of three quarters of what is left (16 to 256 Mi bases) straight
+ * into the batch, and each range of scan tiles whose groups (and the group after them) have landed is
+ * scanned while the next chunk is copied; the rest of the step follows as one graph launch.  Results as after ah_plan_launch.
  * Returns with the work enqueued on the context's stream; the host arrays must stay valid until the
  * stream is synchronised (page-locked memory is fastest).  AH_EINVAL for a group past the batch or a
  * plan over a slice.  The plan's batch is overwritten. */

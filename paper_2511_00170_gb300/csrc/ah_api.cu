@@ -316,7 +316,8 @@ void launch_pieces(ah_ctx* ctx, const Pieces& pieces, uint32_t n, uint64_t g_beg
   if (g_begin >= g_end) return;
   // 8 lanes below 16 groups a piece, else 32.  Groups per window, measured: 200,000 reads of 251 bases
   // with 64 / 32 / 16 / 8 groups 47 / 44 / 48 / 67 us; 20,011 contigs (1.20 Gbp) with 256 / 512 / 1,024 /
-  // 2,048 groups 365 / 329 / 318 / 323 us a call.  Fewer where that leaves SMs without work.
+  // 2,048 groups 365 / 329 / 318 / 323 us a call without its closing wait, which adds 105.  Fewer where that
+  // leaves SMs without work.
   const uint64_t groups = g_end - g_begin;
   const bool narrow = groups < 16ull * n;
   const uint32_t lanes = narrow ? 8 : 32;

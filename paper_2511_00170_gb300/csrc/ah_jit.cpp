@@ -585,8 +585,8 @@ void emit_pattern_tables(std::ostringstream& os, const std::vector<Pattern>& pat
 // survival of 4e-5 per window, against 15 for the exact count of nine positions at 1.6e-4).
 // Surviving words go to a queue per warp and the whole warp checks them after its loop.
 //
-// ALU-bound: about 76 ALU instructions per 32 positions for the bench pair (149 in the shifted form),
-// the pipe 86 % busy (ncu).  Against the shifted form: 1.92 Gbp of random bases, bench pair at k = 3
+// ALU-bound: 80 ALU instructions executed per 32 positions for the bench pair (149 in the shifted form),
+// the pipe 84 % busy (ncu).  Against the shifted form: 1.92 Gbp of random bases, bench pair at k = 3
 // 0.290 ms (0.495), four pairs 0.755 (1.353), eight pairs 1.132 (2.551); the 2,000-genome database
 // (7.61 Gbp, k = 3) 1.087 ms (1.808).  Two warps per block and 18.8 KB of shared memory per warp give
 // 12 warps per SM at up to 168 registers; 16-24 warps with the two code planes in place of one-hot
