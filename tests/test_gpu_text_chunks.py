@@ -223,9 +223,9 @@ def test_fastq_across_chunks(ah_ctx, k, memory):
 def test_fastq_more_records_than_the_first_room(ah_ctx, memory):
     ah, ctx = ah_ctx
     n = 20 << 20
-    text = _fastq(n, borders(n, LEAST), [142], 70, 40)
+    text = _fastq(n, borders(n, LEAST), [142], 70, 15)
     names, seqs, quals = oracle.parse_fastq(text)
-    assert len(borders(n, LEAST)) >= 1 and len(names) > 4096 + n // 256
+    assert len(borders(n, LEAST)) >= 1 and len(names) > 4096 + n // 64
     m = _Memory(text, memory)
     batch, q, got = ah.ah_fastq_pack(ctx, m.ptr, n_bytes=m.n)
     try:
