@@ -559,6 +559,7 @@ void ah_ctx_destroy(ah_ctx* ctx) {
   if (ctx->d_status) cudaFree(ctx->d_status);
   if (ctx->h_status) cudaFreeHost(ctx->h_status);
   if (ctx->h_read) cudaFreeHost(ctx->h_read);
+  if (ctx->emitted) cudaEventDestroy(ctx->emitted);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
 }
@@ -1206,10 +1207,10 @@ ah_status ah_hits_count(const ah_hits* h, uint64_t* n) {
 
 ah_status ah_hits_device(const ah_hits* h, const ah_hit** d_hits, const uint64_t** d_pair_offsets) {
   if (!h) return AH_EINVAL;
-  if (h->written) {  // the caller may read the sites on a stream of its own, also while it captures one
+  if (h->emitted) {  // the caller may read the sites on a stream of its own, also while it captures one
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
-    const cudaError_t e = cudaEventSynchronize(h->written);
+    const cudaError_t e = cudaEventSynchronize(h->ctx->emitted);  // of this scan or a later one
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) return fail(h->ctx, AH_ECUDA, "ah_hits_device: %s", cudaGetErrorString(e));
   }
@@ -1228,7 +1229,6 @@ void ah_hits_free(ah_hits* h) {
   if (!h) return;
   dfree(h->ctx, h->d);
   dfree(h->ctx, h->d_pair_off);
-  if (h->written) cudaEventDestroy(h->written);
   delete h;
 }
 

@@ -128,6 +128,7 @@ struct ah_ctx {
   cudaMemPool_t pool = nullptr;      // the context's stream-ordered memory pool
   uint8_t* bounce[2] = {nullptr, nullptr};       // page-locked buffers for copies into pageable memory
   cudaEvent_t bounce_ev[2] = {nullptr, nullptr};
+  cudaEvent_t emitted = nullptr;     // the end of the last scan's emission (made by the first)
   bool stage_pending = false;        // an upload from bounce[0] may be in flight (its end: bounce_ev[0])
   uint32_t* d_status = nullptr;      // device status word
   uint32_t* h_status = nullptr;      // pinned mirror
@@ -216,7 +217,7 @@ struct ah_hits {
   ah_hit* d = nullptr;
   uint64_t* d_pair_off = nullptr;      // n_pairs + 1
   std::vector<uint64_t> h_pair_off;
-  cudaEvent_t written = nullptr;       // the emission's end where the scan returned before it (ah_hits_device waits)
+  bool emitted = false;                // written by the context's stream before ctx->emitted, which ah_hits_device waits for
 };
 
 struct ah_amplicons {

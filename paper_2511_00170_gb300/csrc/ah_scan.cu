@@ -780,8 +780,9 @@ ah_status scan_sites(ah_ctx* ctx, const ah_batch* b, const ah_primers* p, bool p
     launched(ctx);
     cudaError_t e = cudaGetLastError();
     // the context's own calls are ordered after the emission; a reader on another stream waits for it
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->written, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventRecord(h->written, ctx->stream);
+    if (e == cudaSuccess && !ctx->emitted) e = cudaEventCreateWithFlags(&ctx->emitted, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->emitted, ctx->stream);
+    h->emitted = e == cudaSuccess;
     if (e != cudaSuccess) return done(fail(ctx, AH_ECUDA, "site emission failed: %s", cudaGetErrorString(e)));
   }
   return done(AH_OK);
